@@ -470,7 +470,22 @@ int gdag_launch_external(gdag_ctx *ctx, void (*fn)(void *stream, void *user),
  * placed and issued exactly as its own call would be (gdag_launch,
  * gdag_launch_fused, gdag_array_write with src NULL, or
  * gdag_array_prefetch_host), in order, so the DAG, the streams, the waits
- * and the results are those of the single calls.                         */
+ * and the results are those of the single calls.
+ *
+ * Merged launches: under the PARALLEL policy, with trace = 0, consecutive
+ * launches of built-in kernels (automatic shape, the signature's access
+ * modes) that a merged kernel can do together are issued as one unit, at the
+ * place of its first launch.  Each stays an element of its own, with the same
+ * edges; the unit takes one stream, waits for the parents of all its members
+ * and completes as a whole, so the streams and waits, and the numbering of
+ * the nodes inside the call, may differ from the single calls'.  A launch
+ * joins a unit only if every launch it would overtake touches nothing that it
+ * writes and writes nothing that it touches.  If a unit fails, all its
+ * members fail: *issued counts the elements before its first one, and
+ * nodes_out names the later elements that an earlier unit had issued already.
+ * The units:
+ *   gauss_blur x 2, sobel x 2, minmax x 2, extend x 2, unsharp, combine (the
+ *     IMG program, the second blur the wider one, radii up to 4).           */
 #define GDAG_ELEM_LAUNCH        0  /* gdag_launch                            */
 #define GDAG_ELEM_LAUNCH_FUSED  1  /* gdag_launch_fused                      */
 #define GDAG_ELEM_WRITE         2  /* gdag_array_write(a, NULL, off, bytes):

@@ -120,6 +120,12 @@ class CudaBackend final : public Backend {
         if (e == cudaSuccess) e = cudaGetLastError();
         return chk(e, k.name.c_str());
     }
+    int launch_merged(const Merge &m, const LaunchArgs *const *a, const char *name, void *s) override
+    {
+        cudaError_t e = (cudaError_t)m.launch(a, m.count, s);
+        if (e == cudaSuccess) e = cudaGetLastError();
+        return chk(e, name);
+    }
     int copy_h2d(void *dst, const void *src, size_t bytes, void *s) override
     {
         return chk(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, (cudaStream_t)s), "cudaMemcpyAsync H2D");
@@ -204,6 +210,7 @@ class FakeBackend final : public Backend {
     int stream_query(void *) override { return complete_ == 1 ? BE_OK : BE_NOT_READY; }
     int launch(const KernelEntry &, const LaunchArgs &, void *) override { return op(); }
     int launch_fused(const KernelEntry &, const LaunchArgs *, int, void *) override { return op(); }
+    int launch_merged(const Merge &, const LaunchArgs *const *, const char *, void *) override { return op(); }
     int copy_h2d(void *, const void *, size_t, void *) override { return op(); }
     int copy_d2h(void *, const void *, size_t, void *) override { return op(); }
     int external(void (*fn)(void *, void *), void *user, void *s) override

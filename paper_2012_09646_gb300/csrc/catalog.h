@@ -49,6 +49,31 @@ typedef int (*LauncherFn)(const LaunchArgs &, void *stream);
 // `count` exceeds the kernel's table capacity); returns a cudaError_t value.
 typedef int (*FusedLauncherFn)(const LaunchArgs *members, int count, void *stream);
 
+// Merged launches.  gdag_issue hands a merge rule the run of consecutive
+// built-in launches that starts at a launch of the rule's kernel (each
+// resolved and validated, with its signature's access modes and the automatic
+// launch shape).  The rule may claim several of them, run[0] among them, to be
+// issued as one unit, whose launcher does the work of all members.  The
+// runtime checks that moving the later members up to the first one's place
+// passes no conflicting launch, and that no array that a member writes shares
+// memory with another array of the unit.
+constexpr int kMaxRun = 32;
+
+struct KernelEntry;
+struct RunLaunch {
+    const KernelEntry *k = nullptr;
+    LaunchArgs a;
+    int32_t array[kMaxArgs];  // array handles (array arguments only)
+};
+
+struct Merge {
+    int count = 0;
+    int member[kMaxRun];  // indices into the run, in the order the launcher wants them
+    // as LauncherFn, over the members' arguments
+    int (*launch)(const LaunchArgs *const *m, int count, void *stream) = nullptr;
+};
+typedef bool (*MergeFn)(const RunLaunch *run, int n, Merge &out);
+
 struct KernelEntry {
     std::string name;
     const void *fn = nullptr;  // user kernels: the __global__ handle
@@ -57,6 +82,7 @@ struct KernelEntry {
     ValidateFn validate = nullptr;  // built-ins only
     LauncherFn launcher = nullptr;  // built-ins only
     FusedLauncherFn fused = nullptr;  // built-ins with a fused form only
+    MergeFn merge = nullptr;          // built-ins that start a merged launch only
 };
 
 // Built-in kernels (defined by the kernel translation units).

@@ -534,7 +534,7 @@ int launch_l2norm(const LaunchArgs &a, void *s)
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     // the combine as a programmatic dependent of the partial sums
-    return launch_dependent(l2norm_combine_kernel, kL2CombineThreads, (cudaStream_t)s, (const double *)part,
+    return launch_dependent(l2norm_combine_kernel, 1, kL2CombineThreads, (cudaStream_t)s, (const double *)part,
                             a.p<float>(1), (int)g);
 }
 

@@ -14,52 +14,11 @@
 
 #include "catalog.h"
 #include "kcommon.cuh"
+#include "img.cuh"
 
 namespace gdag {
 
 constexpr int kMaxRadius = 8;
-
-__device__ __forceinline__ int clampi(int v, int lo, int hi) { return v < lo ? lo : (v > hi ? hi : v); }
-
-// Warp-strip stencils.  Each warp owns a strip of image columns, four per
-// lane (one 128-bit load per row and lane), and slides down a band of rows:
-// the vertical taps come from a window of rows kept in registers (each input
-// row is loaded once), the horizontal taps from the neighbouring lanes'
-// registers by warp shuffles, so there is no shared memory and no block
-// barrier.  The HL lanes at each end of a warp are halo lanes: they load
-// and filter the columns next to the strip (replicated at the image edge)
-// but store nothing, so a strip is 4 (32 - 2 HL) columns wide.  Rows and
-// columns outside the image take the nearest edge value (clamp-to-edge).
-constexpr int kStWarps = 4;
-constexpr int kStThreads = 32 * kStWarps;
-constexpr unsigned kFull = 0xffffffffu;
-
-// Pixels x .. x+3 of row y, clamped to the image; one 128-bit load when the
-// four lie inside the image and rows are 16-byte aligned (vec).
-__device__ __forceinline__ float4 load4_clamped(const float *__restrict__ in, int rows, int cols, bool vec, int y, int x)
-{
-    const float *row = in + (size_t)clampi(y, 0, rows - 1) * cols;
-    if (vec && x >= 0 && x + 3 < cols) return __ldg(reinterpret_cast<const float4 *>(row + x));
-    return make_float4(__ldg(row + clampi(x, 0, cols - 1)), __ldg(row + clampi(x + 1, 0, cols - 1)),
-                       __ldg(row + clampi(x + 2, 0, cols - 1)), __ldg(row + clampi(x + 3, 0, cols - 1)));
-}
-
-// Store pixels x .. x+3 (x >= 0) of row y, those inside the image.
-__device__ __forceinline__ void store4(float *__restrict__ out, int rows, int cols, bool vec, int y, int x, float4 v)
-{
-    if (y >= rows || x >= cols) return;
-    float *o = out + (size_t)y * cols + x;
-    if (vec && x + 3 < cols) {
-        *reinterpret_cast<float4 *>(o) = v;
-    } else {
-        o[0] = v.x;
-        if (x + 1 < cols) o[1] = v.y;
-        if (x + 2 < cols) o[2] = v.z;
-        if (x + 3 < cols) o[3] = v.w;
-    }
-}
-
-__device__ __forceinline__ bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 
 // Separable Gaussian blur of radius R.  Per output row a lane makes four
 // outputs: the vertical pass (2R+1 taps on the row window, packed fp32x2
@@ -160,18 +119,6 @@ __global__ void __launch_bounds__(kStThreads) gauss_blur_kernel(const float *__r
     }
 }
 
-// sqrt(gx^2 + gy^2) with the single-instruction approximate square root
-// (relative error about 1e-7, far inside the 1e-5 tolerance; the outputs
-// that are compared bit for bit downstream are min/max of these values
-// themselves); exactly 0 for a flat neighbourhood.
-__device__ __forceinline__ float sobel_mag(float gx, float gy)
-{
-    const float g2 = fmaf(gx, gx, gy * gy);
-    float r;
-    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(g2));
-    return g2 > 0.f ? r : 0.f;
-}
-
 // Sobel magnitude, separably: per column the vertical smoothing
 // sv = top + 2 mid + bottom and difference dv = bottom - top of three rows
 // in registers; gx = sv(c+1) - sv(c-1), gy = dv(c-1) + 2 dv(c) + dv(c+1),
@@ -226,7 +173,6 @@ __global__ void __launch_bounds__(kStThreads) sobel_kernel(const float *__restri
 constexpr int kMmThreads = 128;
 constexpr int kMmV = 16;                      // float4 per thread per chunk
 constexpr int kMmChunk4 = kMmThreads * kMmV;  // 2048 float4
-constexpr int kMmMaxBlocks = 4096;
 constexpr int kMmCombineThreads = 256;
 
 inline unsigned minmax_grid(int64_t n)
@@ -362,8 +308,6 @@ __global__ void __launch_bounds__(1024) extend_kernel(float *__restrict__ x, con
     }
 }
 
-__device__ __forceinline__ float unsharp1(float a, float b, float alpha) { return fmaf(alpha, a - b, a); }
-
 __global__ void __launch_bounds__(1024) unsharp_kernel(const float *__restrict__ img, const float *__restrict__ bl,
                                                        float *__restrict__ out, float alpha, int64_t n)
 {
@@ -399,11 +343,6 @@ __global__ void __launch_bounds__(1024) unsharp_kernel(const float *__restrict__
         for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
             out[i] = unsharp1(img[i], bl[i], alpha);
     }
-}
-
-__device__ __forceinline__ float combine1(float s, float b5, float b9, float e5, float e9)
-{
-    return e5 * s + (1.f - e5) * (e9 * b5 + (1.f - e9) * b9);
 }
 
 __global__ void __launch_bounds__(1024) combine_kernel(const float *__restrict__ s, const float *__restrict__ b5,
@@ -528,7 +467,7 @@ int launch_minmax(const LaunchArgs &a, void *s)
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     // the combine as a programmatic dependent of the block pairs
-    return launch_dependent(minmax_combine_kernel, kMmCombineThreads, (cudaStream_t)s, (const float2 *)part,
+    return launch_dependent(minmax_combine_kernel, 1, kMmCombineThreads, (cudaStream_t)s, (const float2 *)part,
                             a.p<float>(1), (int)g);
 }
 
@@ -603,11 +542,14 @@ KernelEntry entry(const char *name, const void *fn, std::initializer_list<gdag_a
 
 }  // namespace
 
+bool merge_img(const RunLaunch *run, int n, Merge &out);  // k_img_merge.cu
+
 void append_img_kernels(std::vector<KernelEntry> &v)
 {
     v.push_back(entry("gauss_blur", (const void *)gauss_blur_kernel<2>,
                       {arr(GDAG_MODE_IN), arr(GDAG_MODE_OUT), arr(GDAG_MODE_IN), scal(4), scal(4), scal(4)},
                       validate_blur, launch_blur));
+    v.back().merge = merge_img;
     v.push_back(entry("sobel", (const void *)sobel_kernel, {arr(GDAG_MODE_IN), arr(GDAG_MODE_OUT), scal(4), scal(4)},
                       validate_sobel, launch_sobel));
     v.push_back(entry("minmax", (const void *)minmax_kernel,

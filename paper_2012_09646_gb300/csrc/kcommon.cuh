@@ -76,17 +76,17 @@ template <int Width> constexpr size_t reduce_scratch_bytes()
 }
 
 #ifdef __CUDACC__
-// One block of `threads` threads of `kernel` on stream s, launched as a
+// A grid of `threads`-thread blocks of `kernel` on stream s, launched as a
 // programmatic dependent of the kernel before it on s: it may become
 // resident while that kernel runs (once every block of it has executed
 // griddepcontrol.launch_dependents) and must execute griddepcontrol.wait,
 // which returns when that kernel has completed and its writes are visible,
 // before it reads anything that kernel wrote.
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_dependent(void (*kernel)(KArgs...), int threads, cudaStream_t s, Args... args)
+inline cudaError_t launch_dependent(void (*kernel)(KArgs...), dim3 grid, int threads, cudaStream_t s, Args... args)
 {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(1);
+    cfg.gridDim = grid;
     cfg.blockDim = dim3((unsigned)threads);
     cfg.dynamicSmemBytes = 0;
     cfg.stream = s;

@@ -119,6 +119,7 @@ struct Ctx {
     uint64_t tick = 0;
 
     std::vector<void *> events;      // pooled (non-timing)
+    std::vector<int32_t> event_refs; // active nodes holding each (the members of a merged launch share one)
     std::vector<int32_t> free_events;
     std::vector<void *> tevents;     // timing events (trace), never reused
     void *t0 = nullptr;              // trace time base
@@ -219,12 +220,14 @@ struct Ctx {
         if (!free_events.empty()) {
             *slot = free_events.back();
             free_events.pop_back();
+            event_refs[(size_t)*slot] = 1;
             return GDAG_OK;
         }
         void *e;
         int r = be->event_create(&e, false);
         if (r) return be_fail(r, "event create");
         events.push_back(e);
+        event_refs.push_back(1);
         *slot = (int32_t)events.size() - 1;
         return GDAG_OK;
     }
@@ -237,7 +240,7 @@ struct Ctx {
         n->active = false;
         --active_count;
         if (n->event >= 0) {
-            free_events.push_back(n->event);
+            if (--event_refs[(size_t)n->event] == 0) free_events.push_back(n->event);
             n->event = -1;
         }
         if (n->stream >= 0) {
@@ -486,23 +489,29 @@ struct Ctx {
     int retire_done_parents()
     {
         if (!opt.retire_by_query || capturing) return GDAG_OK;
+        // the members of a merged launch share one event: it is asked once
+        int32_t pending = -1, ready = -1;
         for (int64_t p : par) {
             Node *n = node(p);
-            if (!n || !n->active || n->event < 0) continue;
-            int q = be->event_query(events[(size_t)n->event]);
-            if (q == BE_OK) {
-                log_op(GDAG_OP_QUERY_DONE, n->stream, n->event, p);
-                retire(p);
+            if (!n || !n->active || n->event < 0 || n->event == pending) continue;
+            if (n->event != ready) {
+                const int q = be->event_query(events[(size_t)n->event]);
+                if (q == BE_NOT_READY) {
+                    pending = n->event;
+                    continue;
+                }
+                if (q != BE_OK) return be_fail(q, "event query");
+                ready = n->event;
             }
-            else if (q != BE_NOT_READY)
-                return be_fail(q, "event query");
+            log_op(GDAG_OP_QUERY_DONE, n->stream, n->event, p);
+            retire(p);
         }
         return GDAG_OK;
     }
 
-    // Choose the stream, issue waits on active parents of other streams
-    // (only the latest parent per stream), mark the node active there.
-    int place(int64_t id, int32_t *stream_out)
+    // Choose the stream and issue waits on active parents of other streams
+    // (only the latest parent per stream).
+    int choose_and_wait(int32_t *stream_out)
     {
         int r = retire_done_parents();
         if (r) return r;
@@ -534,10 +543,21 @@ struct Ctx {
             r = wait_on(s, latest[k]);
             if (r) return r;
         }
-        Node *me = node(id);
-        me->stream = s;
-        me->active = true;
+        *stream_out = s;
+        return GDAG_OK;
+    }
+
+    // Mark node id active.
+    void activate(int64_t id)
+    {
+        node(id)->active = true;
         ++active_count;
+    }
+
+    // Put the active node id on stream s as its last work.
+    void attach(int64_t id, int32_t s)
+    {
+        node(id)->stream = s;
         StreamState &ss = streams[(size_t)s];
         if (ss.queued) {  // taken from the FIFO by the LRU path: drop it
             ss.queued = false;
@@ -546,7 +566,19 @@ struct Ctx {
         ss.active++;
         ss.tail = id;
         ss.last_use = ++tick;
-        if (opt.record_log == 1) node_log.back().stream = s;
+        if (opt.record_log == 1) node_log[node_log.size() - (size_t)(next_id() - id)].stream = s;
+    }
+
+    // Choose the stream, issue the waits, mark the node active there.
+    int place(int64_t id, int32_t *stream_out)
+    {
+        int32_t s;
+        int r = choose_and_wait(&s);
+        if (r) return r;
+        activate(id);
+        attach(id, s);
+        Node *me = node(id);
+        StreamState &ss = streams[(size_t)s];
         *stream_out = s;
         if (opt.trace) {
             void *e;
@@ -1279,24 +1311,212 @@ int gdag_array_prefetch_host(gdag_ctx *c, gdag_array a, size_t off, size_t bytes
     return c->finish(id, st);
 }
 
-// gdag_issue without the automatic capture: each element as its own call
+// The arguments of launch element i inside the list.
+static bool elem_args_ok(const gdag_elem &e, int64_t nargs_total)
+{
+    const int64_t count = e.type == GDAG_ELEM_LAUNCH ? 1 : (int64_t)e.count;
+    return e.nargs >= 0 && count >= 1 && e.arg0 >= 0 && e.arg0 <= nargs_total &&
+           (int64_t)e.nargs * count <= nargs_total - e.arg0;
+}
+
+// Resolve launch element e for a merge rule: a built-in kernel with the
+// automatic shape and its signature's access modes, valid as it stands.
+// False (with the context's last error restored) ends the run.
+static bool run_launch(gdag_ctx *c, const gdag_elem &e, const gdag_arg *args, int64_t nargs_total,
+                       gdag::RunLaunch &out, Access *acc, int *nacc)
+{
+    if (e.type != GDAG_ELEM_LAUNCH || e.smem || e.grid.x || e.grid.y || e.grid.z || !elem_args_ok(e, nargs_total))
+        return false;
+    if (e.kernel < 0 || (size_t)e.kernel >= c->kernels.size() || !c->kernels[(size_t)e.kernel].launcher) return false;
+    const KernelEntry &k = c->kernels[(size_t)e.kernel];
+    const gdag_arg *a = e.nargs ? args + e.arg0 : nullptr;
+    if (e.nargs != k.nargs) return false;
+    std::fill(out.array, out.array + gdag::kMaxArgs, -1);
+    for (int i = 0; i < e.nargs; ++i) {
+        if (a[i].kind == GDAG_ARG_ARRAY && a[i].mode != GDAG_MODE_SIGNATURE && a[i].mode != k.spec[i].mode) return false;
+        if (a[i].kind == GDAG_ARG_ARRAY) out.array[i] = a[i].array;
+    }
+    const std::string msg = c->last_error;
+    if (resolve(c, e.kernel, e.grid, e.block, 0, a, e.nargs, out.a, acc, nacc)) {
+        c->last_error = msg;
+        return false;
+    }
+    out.k = &k;
+    return true;
+}
+
+static bool conflicting(const Access *a, int na, const Access *b, int nb)
+{
+    for (int i = 0; i < na; ++i)
+        for (int j = 0; j < nb; ++j)
+            if (a[i].array == b[j].array && ((a[i].bits | b[j].bits) & gdag::W_BIT)) return true;
+    return false;
+}
+
+// The run of launches that starts at element i (elements already issued as
+// members of an earlier unit are passed over), and what its first launch's
+// rule makes of it.
+struct MergeRun {
+    gdag::RunLaunch run[gdag::kMaxRun];
+    Access acc[gdag::kMaxRun][gdag::kMaxArgs];
+    int nacc[gdag::kMaxRun];
+    int32_t elem[gdag::kMaxRun];
+    int n = 0;
+    gdag::Merge m;
+    int order[gdag::kMaxRun];  // the members in the run's order
+};
+
+// The checks a rule leaves to the runtime.
+static bool merge_legal(gdag_ctx *c, MergeRun &q)
+{
+    const gdag::Merge &m = q.m;
+    if (m.count < 2 || m.count > q.n || !m.launch) return false;
+    bool in[gdag::kMaxRun] = {};
+    for (int k = 0; k < m.count; ++k) {
+        if (m.member[k] < 0 || m.member[k] >= q.n || in[m.member[k]]) return false;
+        in[m.member[k]] = true;
+    }
+    if (!in[0]) return false;
+    for (int j = 0, k = 0; j < q.n; ++j)
+        if (in[j]) q.order[k++] = j;
+    // a member moves up past every launch between it and the first one
+    for (int k = 1; k < m.count; ++k)
+        for (int j = 0, x = q.order[k]; j < x; ++j)
+            if (!in[j] && conflicting(q.acc[j], q.nacc[j], q.acc[x], q.nacc[x])) return false;
+    // what a member writes shares no memory with any other array of the unit
+    // (other handles may name the same memory: the members would no longer
+    // run one after another on it)
+    for (int k = 0; k < m.count; ++k)
+        for (int x = 0; x < q.nacc[m.member[k]]; ++x) {
+            const Access &w = q.acc[m.member[k]][x];
+            if (!(w.bits & gdag::W_BIT)) continue;
+            const ArrayState &ws = c->arrays[(size_t)w.array];
+            const uintptr_t w0 = (uintptr_t)ws.dev, w1 = w0 + ws.bytes;
+            for (int l = 0; l < m.count; ++l)
+                for (int y = 0; y < q.nacc[m.member[l]]; ++y) {
+                    const int32_t o = q.acc[m.member[l]][y].array;
+                    if (o == w.array) continue;
+                    const ArrayState &os = c->arrays[(size_t)o];
+                    const uintptr_t o0 = (uintptr_t)os.dev, o1 = o0 + os.bytes;
+                    if (w0 < o1 && o0 < w1) return false;
+                }
+        }
+    return true;
+}
+
+// Issue the members of q.m as one unit: every member is an element of its own
+// (its edges are logged and its accesses recorded in the run's order), all of
+// them take one place on one stream, after the waits on the parents of any of
+// them outside the unit, one launch does their work and one event stands for
+// it.  ids receives the members' nodes.
+static int issue_merged(gdag_ctx *c, const MergeRun &q, const gdag_elem *elems, int64_t *ids)
+{
+    const gdag::Merge &m = q.m;
+    const int64_t first = c->next_id();
+    const LaunchArgs *la[gdag::kMaxRun];
+    std::vector<int64_t> ext;  // active parents outside the unit
+    for (int k = 0; k < m.count; ++k) {
+        const int x = q.order[k];
+        la[k] = &q.run[m.member[k]].a;
+        c->capture_note(q.acc[x], q.nacc[x]);
+        const int64_t id = c->next_id();
+        c->infer(id, q.acc[x], q.nacc[x]);
+        for (int64_t p : c->par)
+            if (p < first) ext.push_back(p);
+        for (int i = 0; i < q.nacc[x]; ++i)
+            if (q.acc[x][i].bits & gdag::W_BIT) c->arrays[(size_t)q.acc[x][i].array].host_valid = false;
+        c->push_node(GDAG_NODE_KERNEL);
+        c->node(id)->label = elems[q.elem[x]].kernel;
+        c->activate(id);
+        ids[k] = id;
+    }
+    std::sort(ext.begin(), ext.end());
+    ext.erase(std::unique(ext.begin(), ext.end()), ext.end());
+    c->par = ext;
+    // a failure drops every member, as drop_failed drops one
+    auto drop = [&](int rc, int32_t stream) {
+        const std::string msg = c->last_error;
+        bool done = true;
+        if (!c->capturing && !c->poisoned) {
+            if (stream >= 0) {  // launched but not recorded: wait for its stream
+                c->log_op(GDAG_OP_STREAM_SYNC, stream, -1, -1);
+                ++c->st.host_waits;
+                done = c->poll_stream(stream) == GDAG_OK;
+            } else {
+                for (size_t i = 0; i < ext.size() && done; ++i) done = c->host_wait(ext[i]) == GDAG_OK;
+            }
+        }
+        for (int k = m.count - 1; k >= 0; --k) {
+            if (done) c->retire(ids[k]);
+            else c->deactivate(c->node(ids[k]));
+        }
+        c->last_error = msg;
+        return rc;
+    };
+    int32_t s;
+    int r = c->choose_and_wait(&s);
+    if (r) return drop(r, -1);
+    for (int k = 0; k < m.count; ++k) c->attach(ids[k], s);
+    const int64_t last = ids[m.count - 1];
+    c->log_op(GDAG_OP_LAUNCH, s, -1, last);
+    ++c->st.launches;
+    r = c->be->launch_merged(m, la, q.run[0].k->name.c_str(), c->streams[(size_t)s].handle);
+    if (r) return drop(c->be_fail(r, "merged launch"), -1);
+    r = c->record_end(last, s);
+    if (r) return drop(r, s);
+    const int32_t slot = c->node(last)->event;
+    for (int k = 0; k + 1 < m.count; ++k) c->node(ids[k])->event = slot;
+    c->event_refs[(size_t)slot] = m.count;
+    return GDAG_OK;
+}
+
+// gdag_issue without the automatic capture: each element as its own call,
+// except that under the parallel policy (and with no per-element timing
+// asked for) launches that a merge rule claims are issued as one unit, at the
+// place of the unit's first launch.
 static int issue_each(gdag_ctx *c, const gdag_elem *elems, int32_t n, const gdag_arg *args, int64_t nargs_total,
                       int64_t *nodes_out, int32_t *issued)
 {
     if (issued) *issued = 0;
     if (nodes_out)
         for (int32_t i = 0; i < n; ++i) nodes_out[i] = -1;
+    const bool merging = c->opt.policy == GDAG_POLICY_PARALLEL && !c->opt.trace && !c->poisoned;
+    std::vector<uint8_t> done;  // elements issued as members of an earlier unit
     for (int32_t i = 0; i < n; ++i) {
         const gdag_elem &e = elems[i];
+        if (!done.empty() && done[(size_t)i]) {
+            if (issued) *issued = i + 1;
+            continue;
+        }
+        if (merging && e.type == GDAG_ELEM_LAUNCH && i + 1 < n && e.kernel >= 0 &&
+            (size_t)e.kernel < c->kernels.size() && c->kernels[(size_t)e.kernel].merge) {
+            MergeRun q;
+            for (int32_t j = i; j < n && q.n < gdag::kMaxRun; ++j) {
+                if (!done.empty() && done[(size_t)j]) continue;
+                if (!run_launch(c, elems[j], args, nargs_total, q.run[q.n], q.acc[q.n], &q.nacc[q.n])) break;
+                q.elem[q.n++] = j;
+            }
+            if (q.n > 1 && q.run[0].k->merge(q.run, q.n, q.m) && merge_legal(c, q)) {
+                int64_t ids[gdag::kMaxRun];
+                const int r = issue_merged(c, q, elems, ids);
+                if (done.empty()) done.resize((size_t)n, 0);
+                for (int k = 0; k < q.m.count; ++k) {
+                    done[(size_t)q.elem[q.order[k]]] = 1;
+                    if (nodes_out) nodes_out[q.elem[q.order[k]]] = ids[k];
+                }
+                if (r) return r;
+                if (issued) *issued = i + 1;
+                continue;
+            }
+        }
         const int64_t before = c->next_id();
         int64_t node = -1;
         int r;
         switch (e.type) {
         case GDAG_ELEM_LAUNCH:
         case GDAG_ELEM_LAUNCH_FUSED: {
-            const int64_t count = e.type == GDAG_ELEM_LAUNCH ? 1 : (int64_t)e.count;
-            if (e.nargs < 0 || count < 1 || e.arg0 < 0 || e.arg0 > nargs_total ||
-                (int64_t)e.nargs * count > nargs_total - e.arg0) {
+            if (!elem_args_ok(e, nargs_total)) {
+                const int64_t count = e.type == GDAG_ELEM_LAUNCH ? 1 : (int64_t)e.count;
                 r = c->fail(GDAG_ERR_INVALID, "element %d: arguments [%lld, +%lld) outside the %lld given", i,
                             (long long)e.arg0, (long long)e.nargs * count, (long long)nargs_total);
                 break;

@@ -1,0 +1,170 @@
+"""Merged launches in gdag_issue, on the recording backend (CPU only): which
+programs merge, and that merging leaves the DAG as it is: the same elements
+and edges as the single calls, every conflicting pair ordered."""
+import itertools
+import random
+
+import pytest
+
+from paper_2012_09646_gb300 import gdag as G
+
+ROWS, COLS = 40, 56
+PX = ROWS * COLS
+
+
+class Img:
+    """The ten launches of the IMG program as (kernel, arrays, scalars)."""
+
+    def __init__(self, ctx):
+        at = itertools.count(1)
+        arr = lambda nb: ctx.array(dev=next(at) << 24, nbytes=nb)  # noqa: E731
+        im = lambda: arr(4 * PX)  # noqa: E731
+        self.img, self.b5, self.b9, self.e5, self.e9, self.s, self.out = (im() for _ in range(7))
+        self.mm5, self.mm9 = arr(8), arr(8)
+        sc = G.gdag_scratch_bytes("minmax", PX)
+        self.sc5, self.sc9 = arr(sc), arr(sc)
+        self.w5, self.w9 = arr(20), arr(36)
+
+    def launches(self):
+        return [("gauss_blur", self.img, self.b5, self.w5, ROWS, COLS, 2),
+                ("gauss_blur", self.img, self.b9, self.w9, ROWS, COLS, 4),
+                ("sobel", self.b5, self.e5, ROWS, COLS), ("sobel", self.b9, self.e9, ROWS, COLS),
+                ("minmax", self.e5, self.mm5, self.sc5, PX), ("minmax", self.e9, self.mm9, self.sc9, PX),
+                ("extend", self.e5, self.mm5, PX), ("extend", self.e9, self.mm9, PX),
+                ("unsharp", self.img, self.b5, self.s, 0.5, PX),
+                ("combine", self.s, self.b5, self.b9, self.e5, self.e9, self.out, PX)]
+
+
+DEPS = [(0, 2), (1, 3), (2, 4), (3, 5), (4, 6), (5, 7), (0, 8), (6, 9), (7, 9), (8, 9)]
+
+
+def issue(ctx, seq):
+    p = ctx.program()
+    for k, *args in seq:
+        p.launch(k, *args)
+    before = ctx.stats()["launches"]
+    nodes = p.issue()
+    return nodes, ctx.stats()["launches"] - before
+
+
+def edges_by_position(ctx, nodes):
+    at = {n: i for i, n in enumerate(nodes)}
+    return sorted((at[s], at[d], a, k) for s, d, a, k in ctx.edges())
+
+
+def single(seq_of):
+    ctx = G.Context(backend="fake", record_log=True)
+    nodes = [ctx.launch(k, *a) for k, *a in seq_of(Img(ctx))]
+    e = edges_by_position(ctx, nodes)
+    ctx.close()
+    return e
+
+
+@pytest.mark.parametrize("seed", range(12))
+def test_img_program_in_any_valid_order_is_one_launch(seed):
+    rng = random.Random(seed)
+    order = list(range(10))
+    if seed:
+        while True:
+            rng.shuffle(order)
+            at = {e: i for i, e in enumerate(order)}
+            if all(at[a] < at[b] for a, b in DEPS):
+                break
+    seq_of = lambda g: [g.launches()[i] for i in order]  # noqa: E731
+    ctx = G.Context(backend="fake", record_log=True)
+    nodes, n = issue(ctx, seq_of(Img(ctx)))
+    # a program that starts with its blurs is one unit
+    if order[0] in (0, 1):
+        assert n == 1
+    assert sorted(nodes) == list(range(10))
+    assert edges_by_position(ctx, nodes) == single(seq_of)
+    ctx.close()
+
+
+def variants():
+    """Programs that must stay single launches, each a small change."""
+    def moved(f):
+        def seq(g):
+            L = g.launches()
+            f(g, L)
+            return L
+        return seq
+    yield "raw map read before it is stretched", moved(
+        lambda g, L: L.insert(6, ("unsharp", g.e5, g.img, g.out, 0.5, PX)))
+    yield "second blur not wider", moved(lambda g, L: L.__setitem__(1, ("gauss_blur", g.img, g.b9, g.w5, ROWS, COLS, 2)))
+    yield "other size", moved(lambda g, L: L.__setitem__(3, ("sobel", g.b9, g.e9, ROWS - 1, COLS)))
+    yield "in place unsharp", moved(lambda g, L: (L.__setitem__(8, ("unsharp", g.img, g.b5, g.img, 0.5, PX)),
+                                                  L.__setitem__(9, ("combine", g.img, g.b5, g.b9, g.e5, g.e9, g.out, PX))))
+    yield "result over an input", moved(
+        lambda g, L: L.__setitem__(9, ("combine", g.s, g.b5, g.b9, g.e5, g.e9, g.b5, PX)))
+    yield "stretched by the other range", moved(lambda g, L: L.__setitem__(6, ("extend", g.e5, g.mm9, PX)))
+    yield "explicit access mode", moved(
+        lambda g, L: L.__setitem__(2, ("sobel", G.Mode(g.b5, G.GDAG_MODE_INOUT), g.e5, ROWS, COLS)))
+
+
+@pytest.mark.parametrize("name,seq_of", list(variants()), ids=[n for n, _ in variants()])
+def test_other_programs_stay_as_they_are(name, seq_of):
+    ctx = G.Context(backend="fake", record_log=True)
+    seq = seq_of(Img(ctx))
+    nodes, n = issue(ctx, seq)
+    assert n == len(seq) and nodes == list(range(len(seq)))
+    assert edges_by_position(ctx, nodes) == single(seq_of)
+    ctx.close()
+
+
+def test_arrays_that_share_memory_do_not_merge():
+    ctx = G.Context(backend="fake")
+    g = Img(ctx)
+    g.s = ctx.array(dev=(1 << 24) + 4 * PX - 4, nbytes=4 * PX)  # overlaps img
+    assert issue(ctx, g.launches())[1] == 10
+    ctx.close()
+
+
+@pytest.mark.parametrize("opts", [{"policy": G.GDAG_POLICY_SERIAL_ASYNC}, {"policy": G.GDAG_POLICY_SERIAL_SYNC},
+                                  {"trace": True}])
+def test_serial_and_traced_contexts_do_not_merge(opts):
+    ctx = G.Context(backend="fake", **opts)
+    assert issue(ctx, Img(ctx).launches())[1] == 10
+    ctx.close()
+
+
+@pytest.mark.parametrize("trim", [0, 16])
+def test_events_and_nodes_of_units_are_given_back(trim):
+    """Many steps: a unit's members share one pooled event, retire one by one
+    and leave the table."""
+    ctx = G.Context(backend="fake", retire_by_query=True, fake_complete=True, trim_nodes=trim)
+    g = Img(ctx)
+    for _ in range(300):
+        nodes, n = issue(ctx, g.launches())
+        assert n == 1 and all(ctx.done(v) for v in nodes)
+    assert ctx.stats()["active"] == 0
+    if trim:
+        assert ctx.stats()["held_nodes"] <= 4 * trim
+    ctx.sync()
+    ctx.close()
+
+
+@pytest.mark.parametrize("fail", range(0, 4))
+def test_a_failing_unit_drops_all_its_members(fail):
+    """The unit's wait, launch or record fails: the call reports it, every
+    member is retired, and the program can go on."""
+    ctx = G.Context(backend="fake", fake_fail_op=fail, record_log=True)
+    g = Img(ctx)
+    blocker = ctx.array(dev=1 << 40, nbytes=4 * PX)
+    k = 0
+    try:
+        ctx.launch("unsharp", g.out, blocker, g.b5, 0.5, PX)      # writers of b5 and b9 on two streams
+        k = 1
+        ctx.launch("unsharp", blocker, blocker, g.b9, 0.5, PX)
+        k = 2
+        nodes, n = issue(ctx, g.launches())
+    except G.GdagError as e:
+        assert e.code == G.GDAG_ERR_CUDA
+        if k == 2:
+            assert e.issued == 0 and all(v >= 0 for v in e.nodes)
+            assert all(ctx.done(v) for v in e.nodes)
+    nodes, n = issue(ctx, g.launches())
+    assert n == 1
+    ctx.sync()
+    assert ctx.stats()["active"] == 0
+    ctx.close()
