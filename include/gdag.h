@@ -484,6 +484,8 @@ int gdag_launch_external(gdag_ctx *ctx, void (*fn)(void *stream, void *user),
  * members fail: *issued counts the elements before its first one, and
  * nodes_out names the later elements that an earlier unit had issued already.
  * The units:
+ *   vec_square x 2, vec_reduce_diff of the same two arrays;
+ *   independent bs_call launches of up to 2^21 options each;
  *   gauss_blur x 2, sobel x 2, minmax x 2, extend x 2, unsharp, combine (the
  *     IMG program, the second blur the wider one, radii up to 4).           */
 #define GDAG_ELEM_LAUNCH        0  /* gdag_launch                            */

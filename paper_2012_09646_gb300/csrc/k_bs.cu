@@ -295,6 +295,39 @@ int fused_bs(const LaunchArgs *a, int count, void *s)
     return count <= kFuseSmall ? fused_bs_cap<kFuseSmall>(a, count, s) : fused_bs_cap<kFuseTable>(a, count, s);
 }
 
+int launch_bs_run(const LaunchArgs *const *m, int count, void *s)
+{
+    LaunchArgs a[kMaxRun];
+    for (int i = 0; i < count; ++i) a[i] = *m[i];
+    return fused_bs(a, count, s);
+}
+
+// Independent consecutive bs_call launches of up to kBsMergeMax options each
+// become one fused launch.  A launch costs the host about 5 us, so small books
+// are bound by it: ten of 156253 options take 10 us instead of 50-60, ten of 2e6
+// 25-35 us instead of 60 (steps one after another, of one program or of three in
+// turn).  From about 4e6 options a node the device is the bound, and one launch
+// a book is the quicker form (one program's ten of 1e7: 119 us against 139: the
+// fused form's one wave of blocks has a tail that separate launches fill).
+constexpr int64_t kBsMergeMax = 1 << 21;
+
+bool merge_bs(const RunLaunch *run, int n, Merge &out)
+{
+    out.count = 0;
+    for (int i = 0; i < n; ++i) {
+        if (run[i].k->name != "bs_call" || run[i].a.i64(2) > kBsMergeMax) break;
+        // what a member writes, no other member touches
+        bool apart = run[i].array[0] != run[i].array[1];
+        for (int j = 0; j < i; ++j)
+            apart = apart && run[i].array[1] != run[j].array[0] && run[i].array[1] != run[j].array[1] &&
+                    run[i].array[0] != run[j].array[1];
+        if (!apart) break;
+        out.member[out.count++] = i;
+    }
+    out.launch = launch_bs_run;
+    return out.count > 1;
+}
+
 }  // namespace
 
 void append_bs_kernels(std::vector<KernelEntry> &v)
@@ -313,6 +346,7 @@ void append_bs_kernels(std::vector<KernelEntry> &v)
     e.validate = validate_bs;
     e.launcher = launch_bs;
     e.fused = fused_bs;
+    e.merge = merge_bs;
     v.push_back(e);
 }
 

@@ -1,5 +1,6 @@
 // VEC nodes (Section IV-B, VEC): in-place square and the reduction of the
 // difference of the two squared vectors.
+#include <type_traits>
 #include <vector>
 
 #include "catalog.h"
@@ -100,22 +101,39 @@ __global__ void __launch_bounds__(kThreads) vec_square_fused_kernel(const __grid
     }
 }
 
+// x_i - y_i; SQUARE: of the squares, which replace x_i and y_i (each product
+// rounds on its own, as it does in vec_square).
+template <bool SQUARE, class T> __device__ __forceinline__ float diff1(T *x, T *y, int64_t i)
+{
+    float a = x[i], b = y[i];
+    if constexpr (SQUARE) {
+        a = __fmul_rn(a, a);
+        b = __fmul_rn(b, b);
+        x[i] = a;
+        y[i] = b;
+    }
+    return __fsub_rn(a, b);
+}
+
 // z[0] = sum_i (x_i - y_i).  Per thread: Kahan-compensated fp32; per block:
 // fp64 tree; blocks combined in block order by the last block to arrive.
 // scratch: kReduceMaxBlocks doubles + arrival counter (zero on entry, reset
 // to zero on exit).
 // Block `vb` of a launch of `G` blocks of kThreads threads; the plain kernel
 // passes (blockIdx.x, gridDim.x), the fused one a member's virtual block, so
-// both sum the same elements in the same order.
-__device__ __forceinline__ void reduce_diff_block(const float *__restrict__ x, const float *__restrict__ y,
+// both sum the same elements in the same order.  SQUARE: x and y are squared in
+// place on the way (the merged form of two vec_square launches and this one).
+template <bool SQUARE>
+__device__ __forceinline__ void reduce_diff_block(std::conditional_t<SQUARE, float, const float> *__restrict__ x,
+                                                  std::conditional_t<SQUARE, float, const float> *__restrict__ y,
                                                   float *__restrict__ z, double *scratch, int64_t n, int64_t vb,
                                                   int64_t G, double *sh)
 {
     Kahan acc;
     const bool aligned = ((reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(y)) & 15) == 0;
     if (aligned) {
-        const float4 *x4 = reinterpret_cast<const float4 *>(x);
-        const float4 *y4 = reinterpret_cast<const float4 *>(y);
+        auto *x4 = reinterpret_cast<std::conditional_t<SQUARE, float4, const float4> *>(x);
+        auto *y4 = reinterpret_cast<std::conditional_t<SQUARE, float4, const float4> *>(y);
         const int64_t n4 = n >> 2;
         const int64_t tile = (int64_t)kThreads * kUnroll;
         for (int64_t base = vb * tile; base < n4; base += G * tile) {
@@ -132,19 +150,27 @@ __device__ __forceinline__ void reduce_diff_block(const float *__restrict__ x, c
             for (int k = 0; k < kUnroll; ++k) {
                 int64_t i = base + threadIdx.x + (int64_t)k * kThreads;
                 if (i < n4) {
-                    acc.add(a[k].x - b[k].x);
-                    acc.add(a[k].y - b[k].y);
-                    acc.add(a[k].z - b[k].z);
-                    acc.add(a[k].w - b[k].w);
+                    if constexpr (SQUARE) {
+                        a[k] = make_float4(__fmul_rn(a[k].x, a[k].x), __fmul_rn(a[k].y, a[k].y),
+                                           __fmul_rn(a[k].z, a[k].z), __fmul_rn(a[k].w, a[k].w));
+                        b[k] = make_float4(__fmul_rn(b[k].x, b[k].x), __fmul_rn(b[k].y, b[k].y),
+                                           __fmul_rn(b[k].z, b[k].z), __fmul_rn(b[k].w, b[k].w));
+                        x4[i] = a[k];
+                        y4[i] = b[k];
+                    }
+                    acc.add(__fsub_rn(a[k].x, b[k].x));
+                    acc.add(__fsub_rn(a[k].y, b[k].y));
+                    acc.add(__fsub_rn(a[k].z, b[k].z));
+                    acc.add(__fsub_rn(a[k].w, b[k].w));
                 }
             }
         }
         if (vb == 0 && threadIdx.x < (n & 3)) {
             int64_t i = (n4 << 2) + threadIdx.x;
-            acc.add(x[i] - y[i]);
+            acc.add(diff1<SQUARE>(x, y, i));
         }
     } else {
-        for (int64_t i = vb * kThreads + threadIdx.x; i < n; i += G * kThreads) acc.add(x[i] - y[i]);
+        for (int64_t i = vb * kThreads + threadIdx.x; i < n; i += G * kThreads) acc.add(diff1<SQUARE>(x, y, i));
     }
     double bs = block_sum(acc.value(), sh);
     if (threadIdx.x == 0) scratch[vb] = bs;
@@ -165,7 +191,19 @@ __global__ void __launch_bounds__(kThreads) vec_reduce_diff_kernel(const float *
                                                                     int64_t n)
 {
     __shared__ double sh[kThreads / 32];
-    reduce_diff_block(x, y, z, scratch, n, blockIdx.x, gridDim.x, sh);
+    reduce_diff_block<false>(x, y, z, scratch, n, blockIdx.x, gridDim.x, sh);
+}
+
+// x := x * x, y := y * y, z[0] = sum_i (x_i - y_i) of the squares: the VEC
+// program's three launches in one pass (24 bytes an element become 16, and two
+// launches leave a step that the host waits for: 33 to 29 us at 15625 elements, where copies and
+// latencies are the rest, 77.6 to 75.8 us at 1e6, where the host link is).  The blocks and their
+// order are vec_reduce_diff's, so z is the same bits.
+__global__ void __launch_bounds__(kThreads) vec_square_reduce_kernel(float *__restrict__ x, float *__restrict__ y,
+                                                                     float *__restrict__ z, double *scratch, int64_t n)
+{
+    __shared__ double sh[kThreads / 32];
+    reduce_diff_block<true>(x, y, z, scratch, n, blockIdx.x, gridDim.x, sh);
 }
 
 // Fused form: member m runs its own reduce_grid(n >> 2) virtual blocks
@@ -201,7 +239,7 @@ __global__ void __launch_bounds__(kThreads) vec_reduce_diff_fused_kernel(const _
             first = next;
             next = t.start[m + 1];
         }
-        reduce_diff_block(t.x[m], t.y[m], t.z[m], t.scratch[m], t.n[m], it - first, next - first, sh);
+        reduce_diff_block<false>(t.x[m], t.y[m], t.z[m], t.scratch[m], t.n[m], it - first, next - first, sh);
     }
 }
 
@@ -305,6 +343,39 @@ int fused_reduce_diff(const LaunchArgs *a, int count, void *s)
                                : fused_reduce_diff_cap<kFuseTable>(a, count, s);
 }
 
+// vec_square(x), vec_square(y), vec_reduce_diff(x, y): one launch.
+int launch_square_reduce(const LaunchArgs *const *m, int, void *s)
+{
+    const LaunchArgs &r = *m[2];
+    const int64_t n = r.i64(4);
+    vec_square_reduce_kernel<<<reduce_grid(n >> 2), kThreads, 0, (cudaStream_t)s>>>(
+        r.p<float>(0), r.p<float>(1), r.p<float>(2), r.p<double>(3), n);
+    return cudaGetLastError();
+}
+
+// The run's first launch squares an array that the first vec_reduce_diff after
+// it takes, with the other array's square between.  Every element of both is
+// squared and summed, and the four arrays are different ones.
+bool merge_vec(const RunLaunch *run, int n, Merge &out)
+{
+    int r = 1;
+    while (r < n && run[r].k->name != "vec_reduce_diff") ++r;
+    if (r == n) return false;
+    const int32_t x = run[r].array[0], y = run[r].array[1], z = run[r].array[2], sc = run[r].array[3];
+    const int32_t first = run[0].array[0], other = first == x ? y : x;
+    if ((first != x && first != y) || x == y || z == x || z == y || sc == x || sc == y || sc == z) return false;
+    int q = 1;
+    while (q < r && !(run[q].k->name == "vec_square" && run[q].array[0] == other)) ++q;
+    const int64_t len = run[r].a.i64(4);
+    if (q == r || run[0].a.i64(1) != len || run[q].a.i64(1) != len) return false;
+    out.count = 3;
+    out.member[0] = 0;
+    out.member[1] = q;
+    out.member[2] = r;
+    out.launch = launch_square_reduce;
+    return true;
+}
+
 }  // namespace
 
 void append_vec_kernels(std::vector<KernelEntry> &v)
@@ -318,6 +389,7 @@ void append_vec_kernels(std::vector<KernelEntry> &v)
     e.validate = validate_square;
     e.launcher = launch_square;
     e.fused = fused_square;
+    e.merge = merge_vec;
     v.push_back(e);
 
     KernelEntry r;

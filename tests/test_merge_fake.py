@@ -168,3 +168,96 @@ def test_a_failing_unit_drops_all_its_members(fail):
     ctx.sync()
     assert ctx.stats()["active"] == 0
     ctx.close()
+
+
+def vec_arrays(ctx, n=100):
+    at = itertools.count(1)
+    arr = lambda nb: ctx.array(dev=next(at) << 24, nbytes=nb)  # noqa: E731
+    return arr(4 * n), arr(4 * n), arr(4), arr(G.gdag_scratch_bytes("vec_reduce_diff", n)), arr(4 * n)
+
+
+@pytest.mark.parametrize("name,want,seq", [
+    ("the program", 1, lambda x, y, z, s, w: [("vec_square", x, 100), ("vec_square", y, 100),
+                                              ("vec_reduce_diff", x, y, z, s, 100)]),
+    ("squares swapped", 1, lambda x, y, z, s, w: [("vec_square", y, 100), ("vec_square", x, 100),
+                                                  ("vec_reduce_diff", x, y, z, s, 100)]),
+    ("another launch between", 2, lambda x, y, z, s, w: [("vec_square", x, 100), ("vec_square", w, 100),
+                                                         ("vec_square", y, 100), ("vec_reduce_diff", x, y, z, s, 100)]),
+    ("squared twice", 4, lambda x, y, z, s, w: [("vec_square", x, 100), ("vec_square", x, 100), ("vec_square", y, 100),
+                                                ("vec_reduce_diff", x, y, z, s, 100)]),
+    ("a shorter square", 3, lambda x, y, z, s, w: [("vec_square", x, 100), ("vec_square", y, 99),
+                                                   ("vec_reduce_diff", x, y, z, s, 100)]),
+    ("one square", 2, lambda x, y, z, s, w: [("vec_square", x, 100), ("vec_reduce_diff", x, y, z, s, 100)]),
+    ("one array", 3, lambda x, y, z, s, w: [("vec_square", x, 100), ("vec_square", y, 100),
+                                            ("vec_reduce_diff", x, x, z, s, 100)]),
+    ("sum over an input", 3, lambda x, y, z, s, w: [("vec_square", x, 100), ("vec_square", y, 100),
+                                                    ("vec_reduce_diff", x, y, x, s, 100)]),
+])
+def test_vec_programs(name, want, seq):
+    ctx = G.Context(backend="fake", record_log=True)
+    L = seq(*vec_arrays(ctx))
+    nodes, n = issue(ctx, L)
+    one = G.Context(backend="fake", record_log=True)
+    single_nodes = [one.launch(k, *a) for k, *a in seq(*vec_arrays(one))]
+    assert edges_by_position(ctx, nodes) == edges_by_position(one, single_nodes)
+    # "squared twice": the second square of x is the one that leads the unit
+    assert n == (2 if name == "squared twice" else want)
+    ctx.close()
+    one.close()
+
+
+def test_bs_books_merge_while_independent():
+    n = 1000
+    P = (60.0, 0.1, 0.2, 1.0)
+
+    def seq(ctx):
+        a = [ctx.array(dev=(i + 1) << 24, nbytes=4 * n) for i in range(9)]
+        return [("bs_call", a[0], a[1], n, *P), ("bs_call", a[0], a[2], n - 1, *P),   # one input, two outputs
+                ("bs_call", a[2], a[3], n, *P),                                        # reads an output: a new unit
+                ("bs_call", a[4], a[4], n, *P),                                        # in place: alone
+                ("bs_call", a[5], a[6], n, *P), ("bs_call", a[7], a[6], n, *P)]        # one output twice
+    ctx = G.Context(backend="fake", record_log=True)
+    nodes, k = issue(ctx, seq(ctx))
+    one = G.Context(backend="fake", record_log=True)
+    single_nodes = [one.launch(q, *a) for q, *a in seq(one)]
+    assert edges_by_position(ctx, nodes) == edges_by_position(one, single_nodes)
+    assert k == 5
+    ctx.close()
+    one.close()
+
+
+@pytest.mark.parametrize("seed", range(30))
+def test_random_programs_of_built_in_launches_keep_their_edges(seed):
+    """Random VEC and B&S launches over few arrays, merged wherever a rule
+    claims them: the edges are the single calls'."""
+    rng = random.Random(seed)
+    m = 6
+    plan = []
+    for _ in range(rng.randint(2, 40)):
+        k = rng.choice(["vec_square", "vec_square", "bs_call", "vec_reduce_diff"])
+        plan.append((k, [rng.randrange(m) for _ in range(2)], rng.choice([50, 100, 100]), rng.randrange(2)))
+
+    def seq(ctx):
+        a = [ctx.array(dev=(i + 1) << 24, nbytes=400) for i in range(m)]
+        z = [ctx.array(dev=(i + 20) << 24, nbytes=4) for i in range(2)]
+        s = [ctx.array(dev=(i + 30) << 24, nbytes=G.gdag_scratch_bytes("vec_reduce_diff", 100)) for i in range(2)]
+        out = []
+        for k, (i, j), n, q in plan:
+            if k == "vec_square":
+                out.append((k, a[i], n))
+            elif k == "bs_call":
+                out.append((k, a[i], a[j], n, 60.0, 0.1, 0.2, 1.0))
+            else:
+                out.append((k, a[i], a[j], z[q], s[q], n))
+        return out
+    ctx = G.Context(backend="fake", record_log=True)
+    nodes, k = issue(ctx, seq(ctx))
+    one = G.Context(backend="fake", record_log=True)
+    single_nodes = [one.launch(q, *a) for q, *a in seq(one)]
+    assert sorted(nodes) == list(range(len(plan)))
+    assert edges_by_position(ctx, nodes) == edges_by_position(one, single_nodes)
+    # each element is issued after those it depends on
+    for a, b, _, _ in ctx.edges():
+        assert a < b
+    ctx.close()
+    one.close()
