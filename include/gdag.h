@@ -486,6 +486,9 @@ int gdag_launch_external(gdag_ctx *ctx, void (*fn)(void *stream, void *user),
  * The units:
  *   vec_square x 2, vec_reduce_diff of the same two arrays;
  *   independent bs_call launches of up to 2^21 options each;
+ *   dense_scores x 2 over the same X, rows and feats (up to 10 classes each, or
+ *     any of the CUDA-core shapes);
+ *   row_softmax x 2, argmax_combine of the same two matrices, up to 32768 rows;
  *   gauss_blur x 2, sobel x 2, minmax x 2, extend x 2, unsharp, combine (the
  *     IMG program, the second blur the wider one, radii up to 4).           */
 #define GDAG_ELEM_LAUNCH        0  /* gdag_launch                            */

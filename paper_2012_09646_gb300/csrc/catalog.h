@@ -66,11 +66,12 @@ struct RunLaunch {
     int32_t array[kMaxArgs];  // array handles (array arguments only)
 };
 
+// As LauncherFn, over the members' arguments.
+typedef int (*MergeLaunchFn)(const LaunchArgs *const *m, int count, void *stream);
 struct Merge {
     int count = 0;
     int member[kMaxRun];  // indices into the run, in the order the launcher wants them
-    // as LauncherFn, over the members' arguments
-    int (*launch)(const LaunchArgs *const *m, int count, void *stream) = nullptr;
+    MergeLaunchFn launch = nullptr;
 };
 typedef bool (*MergeFn)(const RunLaunch *run, int n, Merge &out);
 

@@ -33,12 +33,21 @@ constexpr int kMlFeatStep = 8;   // features per lane per load (32 bytes)
 // one step fall into different banks.
 __host__ __device__ constexpr int ml_quarter_stride(int feats, int nc4) { return (feats / kMlQuarters) * nc4 * 4 + 4; }
 
+// One launch's table and result, or two launches' over the same X (blockIdx.y
+// picks one).
+struct ScoreTables {
+    const float *T[2], *bias[2];
+    float *S[2];
+    int classes[2];
+};
+
 template <int NC4>
-__global__ void __launch_bounds__(kMlThreads) dense_scores_kernel(const int *__restrict__ X, const float *__restrict__ T,
-                                                                  const float *__restrict__ bias,
-                                                                  float *__restrict__ S, int rows, int feats,
-                                                                  int classes)
+__global__ void __launch_bounds__(kMlThreads) dense_scores_kernel(const int *__restrict__ X, ScoreTables tb, int rows,
+                                                                  int feats)
 {
+    const float *__restrict__ T = blockIdx.y ? tb.T[1] : tb.T[0], *__restrict__ bias = blockIdx.y ? tb.bias[1] : tb.bias[0];
+    float *__restrict__ S = blockIdx.y ? tb.S[1] : tb.S[0];
+    const int classes = blockIdx.y ? tb.classes[1] : tb.classes[0];
     extern __shared__ float4 smem4[];
     float *st = reinterpret_cast<float *>(smem4);
     const int fq = feats / kMlQuarters;  // features per quarter
@@ -167,9 +176,11 @@ __device__ __forceinline__ void cp_async16(void *dst, const void *src, int src_b
 
 template <int NC4>
 __global__ void __launch_bounds__(kPipeThreads, 2)
-    dense_scores_pipe_kernel(const int *__restrict__ X, const float *__restrict__ T, const float *__restrict__ bias,
-                             float *__restrict__ S, int rows, int feats, int classes)
+    dense_scores_pipe_kernel(const int *__restrict__ X, ScoreTables tb, int rows, int feats)
 {
+    const float *__restrict__ T = blockIdx.y ? tb.T[1] : tb.T[0], *__restrict__ bias = blockIdx.y ? tb.bias[1] : tb.bias[0];
+    float *__restrict__ S = blockIdx.y ? tb.S[1] : tb.S[0];
+    const int classes = blockIdx.y ? tb.classes[1] : tb.classes[0];
     extern __shared__ float4 smem4[];
     unsigned char *xs = reinterpret_cast<unsigned char *>(smem4);
     float *st = reinterpret_cast<float *>(xs + kPipeStages * kPipeStageBytes);
@@ -294,31 +305,74 @@ __global__ void __launch_bounds__(kPipeThreads, 2)
     asm volatile("cp.async.wait_group 0;" ::: "memory");
 }
 
-// Row softmax in place, one thread per row (classes <= 32), max-subtracted.
-__global__ void __launch_bounds__(256) row_softmax_kernel(float *__restrict__ S, int rows, int classes)
+// v := softmax of v[0 .. classes), max-subtracted.
+template <int MAX> __device__ __forceinline__ void softmax_values(float (&v)[MAX], int classes)
 {
-    const int row = blockIdx.x * blockDim.x + threadIdx.x;
-    if (row >= rows) return;
-    float v[32];
-    float *s = S + (size_t)row * classes;
     float m = -INFINITY;
 #pragma unroll
-    for (int c = 0; c < 32; ++c)
-        if (c < classes) {
-            v[c] = s[c];
-            m = fmaxf(m, v[c]);
-        }
+    for (int c = 0; c < MAX; ++c)
+        if (c < classes) m = fmaxf(m, v[c]);
     float z = 0.f;
 #pragma unroll
-    for (int c = 0; c < 32; ++c)
+    for (int c = 0; c < MAX; ++c)
         if (c < classes) {
             v[c] = expf(v[c] - m);
             z += v[c];
         }
     const float inv = 1.0f / z;
 #pragma unroll
+    for (int c = 0; c < MAX; ++c)
+        if (c < classes) v[c] *= inv;
+}
+
+// Row softmax in place, one thread per row (classes <= 32).
+__global__ void __launch_bounds__(256) row_softmax_kernel(float *__restrict__ S, int rows, int classes)
+{
+    const int row = blockIdx.x * blockDim.x + threadIdx.x;
+    if (row >= rows) return;
+    float v[32];
+    float *s = S + (size_t)row * classes;
+#pragma unroll
     for (int c = 0; c < 32; ++c)
-        if (c < classes) s[c] = v[c] * inv;
+        if (c < classes) v[c] = s[c];
+    softmax_values<32>(v, classes);
+#pragma unroll
+    for (int c = 0; c < 32; ++c)
+        if (c < classes) s[c] = v[c];
+}
+
+// row_softmax of S1 and of S2 and argmax_combine of the two in one pass: the
+// same operations on a row's values, which stay in registers between them.
+template <int MAX>
+__global__ void __launch_bounds__(128) softmax_argmax_kernel(float *__restrict__ S1, float *__restrict__ S2,
+                                                             int *__restrict__ labels, int rows, int classes)
+{
+    const int row = blockIdx.x * blockDim.x + threadIdx.x;
+    if (row >= rows) return;
+    float a[MAX], b[MAX];
+    float *s1 = S1 + (size_t)row * classes, *s2 = S2 + (size_t)row * classes;
+#pragma unroll
+    for (int c = 0; c < MAX; ++c)
+        if (c < classes) {
+            a[c] = s1[c];
+            b[c] = s2[c];
+        }
+    softmax_values<MAX>(a, classes);
+    softmax_values<MAX>(b, classes);
+    int best = 0;
+    float bv = a[0] + b[0];
+#pragma unroll
+    for (int c = 0; c < MAX; ++c)
+        if (c < classes) {
+            s1[c] = a[c];
+            s2[c] = b[c];
+            const float v = a[c] + b[c];
+            if (v > bv) {
+                bv = v;
+                best = c;
+            }
+        }
+    labels[row] = best;
 }
 
 // labels[i] = argmax_c (P1[i][c] + P2[i][c]), the lowest c among equals.
@@ -343,6 +397,7 @@ __global__ void __launch_bounds__(256) argmax_combine_kernel(const float *__rest
 // the tcgen05 form (k_ml_tc.cu): classes <= 16, feats a multiple of 64 up to 1024
 bool scores_tc_ok(int feats, int classes);
 int launch_scores_tc(const LaunchArgs &a, cudaStream_t s);
+bool merge_scores(const RunLaunch *run, int n, Merge &out);
 
 namespace {
 
@@ -373,8 +428,22 @@ const char *validate_scores(const LaunchArgs &a)
     return nullptr;
 }
 
-template <int NC4> int scores_pipe_launch(const LaunchArgs &a, cudaStream_t s)
+ScoreTables score_tables(const LaunchArgs *const *m, int count)
 {
+    ScoreTables tb = {};
+    for (int i = 0; i < count; ++i) {
+        tb.T[i] = m[i]->p<float>(1);
+        tb.bias[i] = m[i]->p<float>(2);
+        tb.S[i] = m[i]->p<float>(3);
+        tb.classes[i] = m[i]->i32(6);
+    }
+    return tb;
+}
+
+// `count` (1 or 2) launches that share X, rows, feats and NC4.
+template <int NC4> int scores_pipe_launch(const LaunchArgs *const *m, int count, cudaStream_t s)
+{
+    const LaunchArgs &a = *m[0];
     const int rows = a.i32(4), feats = a.i32(5), classes = a.i32(6);
     static bool configured = false;
     if (!configured) {
@@ -388,16 +457,17 @@ template <int NC4> int scores_pipe_launch(const LaunchArgs &a, cudaStream_t s)
     const int64_t ntiles = ceil_div(rows, kPipeRows), slots = 2 * (int64_t)sm_count();
     const int64_t per = ceil_div(ntiles, slots);
     const int64_t grid = ceil_div(ntiles, per);
-    dense_scores_pipe_kernel<NC4><<<(unsigned)grid, kPipeThreads, pipe_smem(feats, classes), s>>>(
-        a.p<int>(0), a.p<float>(1), a.p<float>(2), a.p<float>(3), rows, feats, classes);
+    dense_scores_pipe_kernel<NC4><<<dim3((unsigned)grid, (unsigned)count), kPipeThreads, pipe_smem(feats, classes), s>>>(
+        a.p<int>(0), score_tables(m, count), rows, feats);
     return cudaGetLastError();
 }
 
-template <int NC4> int scores_launch(const LaunchArgs &a, cudaStream_t s)
+template <int NC4> int scores_launch(const LaunchArgs *const *m, int count, cudaStream_t s)
 {
+    const LaunchArgs &a = *m[0];
     const int rows = a.i32(4), feats = a.i32(5), classes = a.i32(6);
     if (rows == 0) return cudaSuccess;
-    if (use_pipe(feats, classes)) return scores_pipe_launch<NC4>(a, s);
+    if (use_pipe(feats, classes)) return scores_pipe_launch<NC4>(m, count, s);
     const size_t smem = dense_smem(feats, classes);
     // per process: raise the dynamic shared-memory limit once and remember
     // the occupancy of the last table size (no device queries on later
@@ -422,21 +492,29 @@ template <int NC4> int scores_launch(const LaunchArgs &a, cudaStream_t s)
     const int64_t groups = ceil_div(rows, 16 * (kMlThreads / 32));
     int64_t grid = (int64_t)sm_count() * per_sm;
     if (grid > groups) grid = groups;
-    dense_scores_kernel<NC4><<<(unsigned)grid, kMlThreads, smem, s>>>(a.p<int>(0), a.p<float>(1), a.p<float>(2),
-                                                                       a.p<float>(3), rows, feats, classes);
+    dense_scores_kernel<NC4><<<dim3((unsigned)grid, (unsigned)count), kMlThreads, smem, s>>>(
+        a.p<int>(0), score_tables(m, count), rows, feats);
     return cudaGetLastError();
+}
+
+// The CUDA-core forms: the table's padded width picks the instance.
+int launch_scores_cuda(const LaunchArgs *const *m, int count, void *sv)
+{
+    cudaStream_t s = (cudaStream_t)sv;
+    switch (nc4_of(m[0]->i32(6))) {
+    case 1: return scores_launch<1>(m, count, s);
+    case 2: return scores_launch<2>(m, count, s);
+    case 3: return scores_launch<3>(m, count, s);
+    default: return scores_launch<4>(m, count, s);
+    }
 }
 
 int launch_scores(const LaunchArgs &a, void *sv)
 {
     cudaStream_t s = (cudaStream_t)sv;
     if (scores_tc_ok(a.i32(5), a.i32(6))) return launch_scores_tc(a, s);
-    switch (nc4_of(a.i32(6))) {
-    case 1: return scores_launch<1>(a, s);
-    case 2: return scores_launch<2>(a, s);
-    case 3: return scores_launch<3>(a, s);
-    default: return scores_launch<4>(a, s);
-    }
+    const LaunchArgs *m[1] = {&a};
+    return launch_scores_cuda(m, 1, s);
 }
 
 const char *validate_softmax(const LaunchArgs &a)
@@ -476,6 +554,50 @@ int launch_argmax(const LaunchArgs &a, void *s)
     return cudaGetLastError();
 }
 
+int launch_softmax_argmax(const LaunchArgs *const *m, int, void *s)
+{
+    const LaunchArgs &l = *m[2];
+    const int rows = l.i32(3), classes = l.i32(4);
+    if (rows == 0) return cudaSuccess;
+    const unsigned g = (unsigned)ceil_div(rows, 128);
+    if (classes <= 16)
+        softmax_argmax_kernel<16><<<g, 128, 0, (cudaStream_t)s>>>(l.p<float>(0), l.p<float>(1), l.p<int>(2), rows, classes);
+    else
+        softmax_argmax_kernel<32><<<g, 128, 0, (cudaStream_t)s>>>(l.p<float>(0), l.p<float>(1), l.p<int>(2), rows, classes);
+    return cudaGetLastError();
+}
+
+// The softmaxes of two score matrices and the argmax of their sum, up to
+// kTailRows rows: there the launches are what a step costs the host (4097 x 96 x
+// 12, one program: 14.6 us a step against 22.9; 30000 x 1024 x 10: 43.0 against
+// 47.6).  On longer matrices the three launches hide behind the score kernels of
+// other programs' steps, with the softmaxes side by side on two streams (60000 x
+// 1024 x 10, three programs in turn: 44.5 us against 45.4 merged; 100000: 70.7
+// against 71.8).
+constexpr int kTailRows = 32768;
+
+bool merge_softmax(const RunLaunch *run, int n, Merge &out)
+{
+    int r = 1;
+    while (r < n && run[r].k->name != "argmax_combine") ++r;
+    if (r == n) return false;
+    const int32_t s1 = run[r].array[0], s2 = run[r].array[1], lab = run[r].array[2], first = run[0].array[0];
+    const int rows = run[r].a.i32(3), classes = run[r].a.i32(4);
+    if (s1 == s2 || lab == s1 || lab == s2 || (first != s1 && first != s2) || rows > kTailRows) return false;
+    const int32_t other = first == s1 ? s2 : s1;
+    int q = 1;
+    while (q < r && !(run[q].k->name == "row_softmax" && run[q].array[0] == other)) ++q;
+    if (q == r) return false;
+    for (int i : {0, q})
+        if (run[i].a.i32(1) != rows || run[i].a.i32(2) != classes) return false;
+    out.count = 3;
+    out.member[0] = 0;
+    out.member[1] = q;
+    out.member[2] = r;
+    out.launch = launch_softmax_argmax;
+    return true;
+}
+
 KernelEntry entry(const char *name, const void *fn, std::initializer_list<gdag_argspec> spec, ValidateFn v,
                   LauncherFn l)
 {
@@ -492,14 +614,26 @@ KernelEntry entry(const char *name, const void *fn, std::initializer_list<gdag_a
 
 }  // namespace
 
+// Both tables padded to the same width: the two halves of one grid.  X comes
+// from L2 for the second; what is saved is a launch, which bounds the small
+// shapes that these forms mostly see.
+MergeLaunchFn scores_cuda_pair(int feats, int classes0, int classes1)
+{
+    return nc4_of(classes0) == nc4_of(classes1) && use_pipe(feats, classes0) == use_pipe(feats, classes1)
+               ? launch_scores_cuda
+               : nullptr;
+}
+
 void append_ml_kernels(std::vector<KernelEntry> &v)
 {
     v.push_back(entry("dense_scores", (const void *)dense_scores_kernel<3>,
                       {arr(GDAG_MODE_IN), arr(GDAG_MODE_IN), arr(GDAG_MODE_IN), arr(GDAG_MODE_OUT), scal(4), scal(4),
                        scal(4)},
                       validate_scores, launch_scores));
+    v.back().merge = merge_scores;
     v.push_back(entry("row_softmax", (const void *)row_softmax_kernel, {arr(GDAG_MODE_INOUT), scal(4), scal(4)},
                       validate_softmax, launch_softmax));
+    v.back().merge = merge_softmax;
     v.push_back(entry("argmax_combine", (const void *)argmax_combine_kernel,
                       {arr(GDAG_MODE_IN), arr(GDAG_MODE_IN), arr(GDAG_MODE_OUT), scal(4), scal(4)}, validate_argmax,
                       launch_argmax));

@@ -7,7 +7,7 @@ import torch
 
 import datagen
 from paper_2012_09646_gb300 import gdag as G
-from paper_2012_09646_gb300.workloads import BsDag, ImgDag, VecDag, gaussian_weights
+from paper_2012_09646_gb300.workloads import BsDag, ImgDag, MlDag, VecDag, gaussian_weights
 
 pytestmark = pytest.mark.gpu
 
@@ -141,3 +141,87 @@ def test_bs_books_equal_their_launches(n, count, want):
             got.append([t.clone() for t in d.C])
     for a, b in zip(*got):
         assert same_bits(a, b)
+
+
+def run_ml(policy, rows, feats, k1, k2, X, T1, b1, T2, b2):
+    """Two score launches over one X (each its own classes); the scores."""
+    with G.Context(policy=policy) as ctx:
+        dev = [torch.as_tensor(np.ascontiguousarray(t)).cuda() for t in (X, T1, b1, T2, b2)]
+        a = [ctx.array(t) for t in dev]
+        S = [torch.full((rows, k), -1.0, device="cuda") for k in (k1, k2)]
+        s = [ctx.array(t) for t in S]
+        torch.cuda.synchronize()
+        p = ctx.program()
+        p.launch("dense_scores", a[0], a[1], a[2], s[0], rows, feats, k1)
+        p.launch("dense_scores", a[0], a[3], a[4], s[1], rows, feats, k2)
+        n = launches(ctx, p.issue)
+        return [t.clone() for t in S], n
+
+
+# the tensor-core pair: one row, the tile's edges, more tiles than SMs; one
+# stage per team and the longest rows; class counts that differ.  The CUDA-core
+# halves: both forms, one padded width.  Last: forms that stay apart
+@pytest.mark.parametrize("rows,feats,k1,k2,want", [
+    (1, 64, 10, 10, 1), (127, 128, 1, 10, 1), (128, 1024, 10, 3, 1), (129, 192, 7, 10, 1), (19457, 64, 10, 10, 1),
+    (20000, 1024, 9, 10, 1), (1, 32, 10, 9, 1), (4097, 96, 12, 10, 1), (300, 992, 12, 12, 1), (301, 992, 16, 13, 1),
+    (100, 128, 10, 11, 2), (100, 96, 12, 8, 2)])
+@pytest.mark.parametrize("values", ["recipe", "general", "wide"])
+def test_two_score_launches_equal_single_ones(rows, feats, k1, k2, want, values):
+    g = np.random.default_rng(rows + feats)
+    X, T1, b1, _, _ = datagen.ml_inputs(rows, feats=feats, classes=k1, seed=1)
+    _, _, _, T2, b2 = datagen.ml_inputs(rows, feats=feats, classes=k2, seed=2)
+    if values == "general":  # tables whose three pieces are all needed
+        T1, T2 = (g.normal(0, 1, t.shape).astype(np.float32) for t in (T1, T2))
+        X = g.integers(-256, 257, X.shape).astype(np.int32)
+    if values == "wide":     # integers that bfloat16 cannot hold, in the first and last rows
+        X = X.copy()
+        X[0, 0], X[-1, -1] = 257, -70000
+    merged, n = run_ml(G.GDAG_POLICY_PARALLEL, rows, feats, k1, k2, X, T1, b1, T2, b2)
+    single, m = run_ml(G.GDAG_POLICY_SERIAL_ASYNC, rows, feats, k1, k2, X, T1, b1, T2, b2)
+    assert (n, m) == (want, 2)
+    for a, b in zip(merged, single):
+        assert same_bits(a, b)
+
+
+@pytest.mark.parametrize("rows,classes,want", [(1, 1, 1), (127, 2, 1), (129, 10, 1), (1000, 16, 1), (513, 17, 1),
+                                               (4097, 32, 1), (32768, 10, 1), (32769, 10, 3)])
+@pytest.mark.parametrize("swap", [False, True])
+def test_softmaxes_and_labels_equal_their_launches(rows, classes, want, swap):
+    g = np.random.default_rng(rows)
+    S = [(g.normal(0, 9, (rows, classes)) + 0.0).astype(np.float32) for _ in range(2)]
+    S[0][0, :] = S[1][0, :] = 0.0                    # ties: the lowest class
+    if rows > 100:
+        S[0][5, 0], S[1][7, classes - 1] = np.nan, np.inf
+    got = []
+    for policy in (G.GDAG_POLICY_PARALLEL, G.GDAG_POLICY_SERIAL_ASYNC):
+        with G.Context(policy=policy) as ctx:
+            t = [torch.from_numpy(s.copy()).cuda() for s in S]
+            lab = torch.full((rows,), -1, dtype=torch.int32, device="cuda")
+            a = [ctx.array(x) for x in t]
+            L = ctx.array(lab)
+            torch.cuda.synchronize()
+            p = ctx.program()
+            for x in (a[::-1] if swap else a):
+                p.launch("row_softmax", x, rows, classes)
+            p.launch("argmax_combine", a[0], a[1], L, rows, classes)
+            n = launches(ctx, p.issue)
+            assert n == (want if policy == G.GDAG_POLICY_PARALLEL else 3)
+            got.append([x.clone() for x in t] + [lab.clone()])
+    for a, b in zip(got[0][:2], got[1][:2]):
+        assert same_bits(torch.nan_to_num(a, nan=7.0), torch.nan_to_num(b, nan=7.0))
+    assert torch.equal(got[0][2], got[1][2])
+
+
+def test_ml_program_equals_its_launches():
+    rows = 5000
+    inp = datagen.ml_inputs(rows, feats=256, classes=10, seed=4)
+    got = []
+    for policy, want in ((G.GDAG_POLICY_PARALLEL, 2), (G.GDAG_POLICY_SERIAL_ASYNC, 5)):
+        with G.Context(policy=policy) as ctx:
+            m = MlDag(ctx, rows, 256, 10)
+            m.load(*inp)
+            for _ in range(3):
+                assert launches(ctx, m.launch_all) == want
+            got.append([t.clone() for t in (m.S1, m.S2, m.labels)])
+    for a, b in zip(*got):
+        assert torch.equal(a, b)

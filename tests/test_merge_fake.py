@@ -261,3 +261,34 @@ def test_random_programs_of_built_in_launches_keep_their_edges(seed):
         assert a < b
     ctx.close()
     one.close()
+
+
+def test_score_and_softmax_programs():
+    """The classifier ensemble: which launches merge, by shape and wiring."""
+    r, f, k = 1000, 128, 10
+
+    def ml(ctx, rows=r, feats=f, c1=k, c2=k, same_x=True, same_s=False, out_over_x=False):
+        at = itertools.count(1)
+        arr = lambda nb: ctx.array(dev=next(at) << 30, nbytes=nb)  # noqa: E731
+        X, X2 = arr(4 * rows * feats), arr(4 * rows * feats)
+        T1, T2, b1, b2 = arr(4 * feats * c1), arr(4 * feats * c2), arr(4 * c1), arr(4 * c2)
+        S1, S2, L = arr(4 * rows * c1), arr(4 * rows * c2), arr(4 * rows)
+        S2 = S1 if same_s else X if out_over_x else S2
+        seq = [("dense_scores", X, T1, b1, S1, rows, feats, c1),
+               ("dense_scores", X if same_x else X2, T2, b2, S2, rows, feats, c2)]
+        if c1 == c2:
+            seq += [("row_softmax", S1, rows, c1), ("row_softmax", S2, rows, c2),
+                    ("argmax_combine", S1, S2, L, rows, c1)]
+        return seq
+
+    for kw, want in (({}, 2), ({"rows": 40000}, 4), ({"c1": 11, "c2": 11}, 3), ({"feats": 96, "c1": 12, "c2": 12}, 2),
+                     ({"feats": 96, "c1": 12, "c2": 4}, 2), ({"c1": 3}, 1), ({"same_x": False}, 3),
+                     ({"same_s": True}, 5), ({"out_over_x": True}, 3)):
+        ctx = G.Context(backend="fake", record_log=True)
+        nodes, n = issue(ctx, ml(ctx, **kw))
+        one = G.Context(backend="fake", record_log=True)
+        single_nodes = [one.launch(q, *a) for q, *a in ml(one, **kw)]
+        assert edges_by_position(ctx, nodes) == edges_by_position(one, single_nodes), kw
+        assert n == want, (kw, n)
+        ctx.close()
+        one.close()
