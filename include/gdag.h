@@ -491,6 +491,7 @@ int gdag_launch_external(gdag_ctx *ctx, void (*fn)(void *stream, void *user),
  *   row_softmax x 2, argmax_combine of the same two matrices, up to 32768 rows;
  *   two independent launches of spmv_csr (up to 2^22 rows and nonzeros each), or
  *     of l2norm, scale, seg_l2norm or seg_scale (up to 2^20 elements each);
+ *   two independent launches of conv3x3_relu_pool or of avgpool_global;
  *   gauss_blur x 2, sobel x 2, minmax x 2, extend x 2, unsharp, combine (the
  *     IMG program, the second blur the wider one, radii up to 4).           */
 #define GDAG_ELEM_LAUNCH        0  /* gdag_launch                            */

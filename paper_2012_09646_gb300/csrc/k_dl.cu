@@ -7,7 +7,7 @@
 //   concat_dense       out = [e1 e2] wd + bd, fp32
 //
 // conv3x3_relu_pool is an implicit GEMM on a persistent grid of one
-// 416-thread CTA per SM that holds all 512 tensor-memory columns: two sets of
+// 576-thread CTA per SM that holds all 512 tensor-memory columns: two sets of
 // accumulators, so that the tensor cores fill one set while the epilogue
 // drains the other.  A tile is two input rows x 256 input columns of one
 // image; its 512 pixels form four M = 128 operands, one per position in the
@@ -16,7 +16,8 @@
 // x0/2 + m and the pooling maximum is taken inside one thread, with no
 // exchange.  N = 64 output channels, K = 27 taps padded to 32, fp32
 // accumulation in tensor memory (four 128-lane x 64-column accumulators per
-// set).
+// set).  A launch does one convolution, or the two of a merged launch, whose
+// tiles follow one another in one grid.
 //
 // K order.  A thread builds its im2col row from three aligned 32-bit words of
 // each staged input row: L = columns (2m-2, 2m-1), C = (2m, 2m+1) and
@@ -31,29 +32,36 @@
 // the canonical K-major layout without swizzle (8-row x 16-byte core
 // matrices, 128 B between K-adjacent and 512 B between M/N-adjacent ones).
 //
-// Warp roles, per tile t (set s = t % 2):
-//   warp 0 (control, one lane): keeps the halo copies (3 channels x 4 rows x
+// Warp roles, per tile t (set s = t % 2).  What bounds a tile is the latency of the
+// chain that it goes through in each role, not a rate, so the producers and the
+// epilogue work in two teams, one per set: each has two tiles' time for its chain.
+//   warp 17 (loader, one lane): keeps the halo copies (3 channels x 4 rows x
 //     272 columns per tile, two cp.async.bulk.tensor boxes, zeros outside
 //     the image, box slots padded to 128-byte boundaries) eight tiles ahead
-//     in a ring of buffers, each completing on its own mbarrier; once the
-//     producers have written A set s ("A full") and the epilogue has
-//     drained accumulator set s ("empty", tile t-2), issues eight
+//     in a ring of buffers, each completing on its own mbarrier, and refills a
+//     buffer once its producers have read it ("halo empty").
+//   warps 1-4 and 5-8 (producers, team s): wait for the tile's halo and for the
+//     MMAs of tile t-2 to have read A set s, build A set s (thread m writes row m
+//     of the four operands), and arrive on "A full" and "halo empty", one arrival
+//     per warp.
+//   warp 0 (control, one lane): once A set s is written ("A full") and the
+//     epilogue has drained accumulator set s ("empty", tile t-2), issues eight
 //     tcgen05.mma.cta_group::1.kind::f16 (K = 16 each) and commits them to
 //     the set's "full" mbarrier.
-//   warps 1-4 (producers): wait for the tile's halo and for the MMAs of tile
-//     t-2 to have read A set s, build A set s (thread m writes row m of the
-//     four operands), and arrive on "A full", one arrival per warp.
-//   warps 5-12 (epilogue): stage the weights once (one round of loads of the
-//     raw weights and bias into a staging buffer, then the two B operands
-//     in the K order, one 16-byte core-matrix row per store); per tile wait
-//     for "full", read the accumulators with
-//     tcgen05.ld (warp w reads lanes 32*(w%4).. and channels 32*((w-5)/4)..),
+//   warps 9-12 and 13-16 (epilogue, team s): all stage the weights once (one round
+//     of loads of the raw weights and bias into a staging buffer, then the two B
+//     operands of each convolution in the K order, one 16-byte core-matrix row per
+//     store); per tile wait for "full", read the accumulators with
+//     tcgen05.ld (warp w reads lanes 32*(w%4).., 16 channels a round),
 //     signal "empty", take the maximum of the four (bias included; ReLU
 //     commutes with the maximum), convert channel pairs to bf16 with ReLU in
-//     one instruction and stage the pooled tile (64 channels x 128 columns,
-//     double-buffered) in shared memory, from where one thread writes it
-//     with one TMA tensor store (8-byte vector stores by all 256 threads when
-//     a pooled row is not a multiple of 8 values).
+//     one instruction and stage the pooled tile (64 channels x 128 columns, two
+//     buffers a team) in shared memory, from where one thread writes it
+//     with one TMA tensor store (8-byte vector stores by the team's 128 threads
+//     when a pooled row is not a multiple of 8 values).
+// Two convolutions of 16 x 3 x 256 x 256 take 22.4 us (0.68 us a tile beside about
+// 4 us of start-up), from 34.4 us as two launches of a form with one team in each
+// role, the halo copies issued by the control lane, and 1.0 us a tile.
 // Every wait is bounded (about one second) and also ends when another role
 // raises the shared abort flag; a warp or role decides to stop with a vote
 // (__all_sync, or a barrier that ANDs its threads' results), so no barrier is
@@ -75,10 +83,12 @@
 namespace gdag {
 
 constexpr int kConvM = 128, kConvN = 64, kConvK = 32, kConvTaps = 27;
-constexpr int kCtlThreads = 32;                      // warp 0: halo copies and MMA issue (one lane)
-constexpr int kProdThreads = 128;                    // warps 1-4: im2col
-constexpr int kEpiThreads = 256;                     // warps 5-12: epilogue and stores
-constexpr int kConvThreads = kCtlThreads + kProdThreads + kEpiThreads;
+constexpr int kCtlThreads = 32;                      // warp 0: MMA issue (one lane)
+constexpr int kTeamThreads = 128;                    // a team of producers or of the epilogue
+constexpr int kProdThreads = 2 * kTeamThreads;       // warps 1-8: im2col
+constexpr int kEpiThreads = 2 * kTeamThreads;        // warps 9-16: epilogue and stores
+constexpr int kLoadThreads = 32;                     // warp 17: halo copies (one lane)
+constexpr int kConvThreads = kCtlThreads + kProdThreads + kEpiThreads + kLoadThreads;
 constexpr int kTileCols = 256;                       // input columns per tile
 constexpr int kHaloBox = 136;                        // columns per TMA box (two boxes: x0-8 .. x0+263)
 constexpr int kHaloBoxBytes = kHaloBox * 4 * 3 * 2;  // 3 channels x 4 rows, bf16: the bytes one box moves
@@ -92,22 +102,36 @@ constexpr int kAccCols = 4 * kConvN;                 // one accumulator set: 256
 constexpr int kTmemCols = 2 * kAccCols;              // two sets: the SM's 512 columns
 constexpr int kStageBytes = kConvN * (kTileCols / 2) * 2;  // pooled tile [64][128] bf16
 constexpr int kOffB = 2 * kOpASet;
-constexpr int kOffHalo = kOffB + 2 * kOpBBytes;
+constexpr int kOpBConv = 2 * kOpBBytes;              // the two B operands of one convolution
+constexpr int kOffHalo = kOffB + 2 * kOpBConv;
 constexpr int kOffStage = kOffHalo + kHaloBufs * kHaloBytes;
-constexpr int kOffBars = kOffStage + 2 * kStageBytes;
-// halo full x kHaloBufs, A full x2, accumulator full x2, accumulator empty x2
-constexpr int kNumBars = kHaloBufs + 6;
-constexpr size_t kConvSmemUsed = kOffBars + kNumBars * 8 + 16;
-// requested dynamic shared memory: more than half of the SM's 228 KB, so that
-// one CTA (holding all 512 tensor-memory columns) owns an SM
-constexpr size_t kConvSmem = 160 * 1024;
-static_assert(kConvSmemUsed <= kConvSmem, "conv shared memory");
+constexpr int kOffBars = kOffStage + 4 * kStageBytes;
+// halo full and halo empty x kHaloBufs, A full x2, accumulator full x2, accumulator empty x2
+constexpr int kNumBars = 2 * kHaloBufs + 6;
+// more than half of the SM's 228 KB, so that one CTA (holding all 512
+// tensor-memory columns) owns an SM
+constexpr size_t kConvSmem = kOffBars + kNumBars * 8 + 16;
+static_assert(kConvSmem > 114 * 1024 && kConvSmem <= 227 * 1024, "conv shared memory");
 static_assert(kConvSmem < (size_t)(0x4000 << 4), "shared addresses fit a matrix descriptor's 14-bit start field");
 static_assert(2 * kConvN * kConvTaps + 4 * kConvN <= kStageBytes, "raw weights must fit one staging buffer");
 static_assert((2 * kConvN * (kConvK / 8)) % kEpiThreads == 0, "B rows split evenly over the epilogue");
 static_assert(kOffHalo % 128 == 0 && kHaloBoxStride % 128 == 0 && kHaloBytes % 128 == 0 && kOffStage % 128 == 0 &&
                   kStageBytes % 128 == 0 && (kHaloBox * 2) % 16 == 0,
               "TMA shared-memory addresses must be 128-byte aligned, box rows multiples of 16 bytes");
+
+// One convolution of a launch.
+struct Conv {
+    CUtensorMap tin, tout;
+    const __nv_bfloat16 *wt;
+    const float *bias;
+    __nv_bfloat16 *out;
+    int *status;
+    int h, w, tma_store;
+    int tiles_x, rows2, ntiles;
+};
+struct ConvPair {
+    Conv m[2];
+};
 
 // byte offset of (row, k) in the canonical K-major, no-swizzle layout
 __device__ __forceinline__ int umma_off(int row, int k)
@@ -157,62 +181,121 @@ __device__ __forceinline__ void conv_tile_coords(int tile, int tiles_x, int rows
 // image*3 + channel); the hardware fills zeros outside the image, including
 // the negative first column and row.  Issued by one thread; completion is
 // counted in bytes on `bar`.
-__device__ __forceinline__ void conv_issue_halo(const CUtensorMap *tin, unsigned char *dst, uint32_t bar, int tile,
-                                                int tiles_x, int rows2)
+__device__ __forceinline__ void conv_issue_halo(const Conv &m, unsigned char *dst, uint32_t bar, int tile)
 {
     int b, y0, x0;
-    conv_tile_coords(tile, tiles_x, rows2, b, y0, x0);
+    conv_tile_coords(tile, m.tiles_x, m.rows2, b, y0, x0);
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(2 * kHaloBoxBytes) : "memory");
 #pragma unroll
     for (int half = 0; half < 2; ++half)
         asm volatile(
             "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(
                 smem_addr(dst + half * kHaloBoxStride)),
-            "l"(reinterpret_cast<uint64_t>(tin)), "r"(x0 - 8 + half * kHaloBox), "r"(y0 - 1), "r"(3 * b), "r"(bar)
+            "l"(reinterpret_cast<uint64_t>(&m.tin)), "r"(x0 - 8 + half * kHaloBox), "r"(y0 - 1), "r"(3 * b), "r"(bar)
             : "memory");
 }
 
+// The raw weights and bias of one convolution into `raw` (one round of loads),
+// then the two B operands in the K order from there, one 16-byte core-matrix row
+// (eight K positions of one channel) per store.  Thread etid builds the rows
+// of channel etid % 64 at K chunk etid / 64 (uniform over a warp) for both
+// parities: the chunk is matched against compile-time values, so every tap
+// index is a constant.
+constexpr int kRawWeights = kConvN * kConvTaps;
+constexpr int kRawPer = (kRawWeights + kEpiThreads - 1) / kEpiThreads;
+__device__ __forceinline__ void conv_load_raw(const Conv &m, unsigned char *raw, int etid)
+{
+    uint16_t *wraw = reinterpret_cast<uint16_t *>(raw);
+    float *braw = reinterpret_cast<float *>(raw + 2 * kRawWeights);
+    const unsigned short *wsrc = reinterpret_cast<const unsigned short *>(m.wt);
+    unsigned short wl[kRawPer];
+#pragma unroll
+    for (int r = 0; r < kRawPer; ++r) {
+        const int i = etid + r * kEpiThreads;
+        wl[r] = i < kRawWeights ? __ldg(wsrc + i) : (unsigned short)0;
+    }
+    const float bl = etid < kConvN ? __ldg(m.bias + etid) : 0.f;
+#pragma unroll
+    for (int r = 0; r < kRawPer; ++r) {
+        const int i = etid + r * kEpiThreads;
+        if (i < kRawWeights) wraw[i] = wl[r];
+    }
+    if (etid < kConvN) braw[etid] = bl;
+}
 
-__global__ void __launch_bounds__(kConvThreads, 1)
-    conv3x3_relu_pool_kernel(const __grid_constant__ CUtensorMap tin, const __grid_constant__ CUtensorMap tout,
-                             const __nv_bfloat16 *__restrict__ wt, const float *__restrict__ bias,
-                             __nv_bfloat16 *__restrict__ out, int *status, int n, int h, int w, int tma_store)
+__device__ __forceinline__ void conv_build_b(const unsigned char *raw, unsigned char *sb, int etid)
+{
+    const uint16_t *wraw = reinterpret_cast<const uint16_t *>(raw);
+    const float *braw = reinterpret_cast<const float *>(raw + 2 * kRawWeights);
+    constexpr int kKc = kConvK / 8;
+    static_assert(kEpiThreads == kConvN * kKc, "one channel and K chunk per epilogue thread");
+    const int co = etid % kConvN, kq = etid / kConvN;
+    const float bb = braw[co];
+    const __nv_bfloat16 bhi = __float2bfloat16_rn(bb);
+    const uint32_t bias_hi = __bfloat16_as_ushort(bhi);
+    const uint32_t bias_lo = __bfloat16_as_ushort(__float2bfloat16_rn(bb - __bfloat162float(bhi)));
+#pragma unroll
+    for (int kc = 0; kc < kKc; ++kc) {
+        if (kc != kq) continue;
+#pragma unroll
+        for (int p = 0; p < 2; ++p) {
+            uint32_t q[4];
+#pragma unroll
+            for (int j = 0; j < 8; j += 2) {
+                uint32_t two = 0;
+#pragma unroll
+                for (int h2 = 0; h2 < 2; ++h2) {
+                    const int k = 8 * kc + j + h2, tap = conv_tap(p, k);
+                    const uint32_t v = tap >= 0 ? (uint32_t)wraw[co * kConvTaps + tap]
+                                                : (k == 27 ? bias_hi : (k == 28 ? bias_lo : 0u));
+                    two |= v << (16 * h2);
+                }
+                q[j / 2] = two;
+            }
+            *reinterpret_cast<uint4 *>(sb + p * kOpBBytes + umma_off(co, 8 * kc)) = make_uint4(q[0], q[1], q[2], q[3]);
+        }
+    }
+}
+
+__global__ void __launch_bounds__(kConvThreads, 1) conv3x3_relu_pool_kernel(const __grid_constant__ ConvPair pair)
 {
     extern __shared__ __align__(1024) unsigned char conv_smem[];
     unsigned char *sa = conv_smem;                  // two sets of four A operands
-    unsigned char *sb = conv_smem + kOffB;          // two B operands
-    unsigned char *halo = conv_smem + kOffHalo;     // two halo buffers [box][ci][row][136]
-    unsigned char *stage = conv_smem + kOffStage;   // two pooled tiles [64][128]
+    unsigned char *sb = conv_smem + kOffB;          // two B operands of each convolution
+    unsigned char *halo = conv_smem + kOffHalo;     // halo buffers [box][ci][row][136]
+    unsigned char *stage = conv_smem + kOffStage;   // two pooled tiles [64][128] a team
     uint64_t *bars = reinterpret_cast<uint64_t *>(conv_smem + kOffBars);
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + kNumBars);
     volatile int *abort = reinterpret_cast<volatile int *>(tmem_slot + 1);
+    const int n0 = pair.m[0].ntiles, ntiles = n0 + pair.m[1].ntiles;
 
     // the TMA copies need a 128-byte aligned window: check before any copy
     // or tensor-memory use (uniform over the CTA)
     if ((smem_addr(conv_smem) & 127u) != 0) {
-        if (threadIdx.x == 0) atomicExch(status, 2);
+        if (threadIdx.x == 0)
+            for (int q = 0; q < 2; ++q)
+                if (pair.m[q].ntiles > 0) atomicExch(pair.m[q].status, 2);
         return;
     }
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int tiles_x = (w + kTileCols - 1) / kTileCols, rows2 = h / 2;
-    const int ntiles = n * rows2 * tiles_x;
-    const int ho = h / 2, wo = w / 2;
-    const uint32_t halo_bar = smem_addr(&bars[0]);  // + 8 * buffer: the tile's halo landed
-    const uint32_t afull_bar = smem_addr(&bars[kHaloBufs]);      // + 8 * set: A written (and the halo read)
-    const uint32_t full_bar = smem_addr(&bars[kHaloBufs + 2]);   // + 8 * set: MMAs done (A read, accumulators ready)
-    const uint32_t empty_bar = smem_addr(&bars[kHaloBufs + 4]);  // + 8 * set: epilogue done reading the accumulators
+    const uint32_t halo_bar = smem_addr(&bars[0]);                // + 8 * buffer: the tile's halo landed
+    const uint32_t hempty_bar = smem_addr(&bars[kHaloBufs]);      // + 8 * buffer: the producers read it
+    const uint32_t afull_bar = smem_addr(&bars[2 * kHaloBufs]);   // + 8 * set: A written
+    const uint32_t full_bar = afull_bar + 16;                     // + 8 * set: MMAs done (A read, accumulators ready)
+    const uint32_t empty_bar = afull_bar + 32;                    // + 8 * set: epilogue done reading the accumulators
 
     if (warp == 0) {
         if (lane == 0) {
             *abort = 0;
-            asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tin)) : "memory");
-            for (int j = 0; j < kHaloBufs; ++j) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(halo_bar + 8 * j));
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(afull_bar), "r"(kProdThreads / 32));
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(afull_bar + 8), "r"(kProdThreads / 32));
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(full_bar));
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(full_bar + 8));
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(empty_bar), "r"(kEpiThreads / 32));
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(empty_bar + 8), "r"(kEpiThreads / 32));
+            for (int j = 0; j < kHaloBufs; ++j) {
+                asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(halo_bar + 8 * j));
+                asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(hempty_bar + 8 * j), "r"(kTeamThreads / 32));
+            }
+            for (int s = 0; s < 2; ++s) {
+                asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(afull_bar + 8 * s), "r"(kTeamThreads / 32));
+                asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(full_bar + 8 * s));
+                asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(empty_bar + 8 * s), "r"(kTeamThreads / 32));
+            }
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         }
         __syncwarp();
@@ -224,38 +307,21 @@ __global__ void __launch_bounds__(kConvThreads, 1)
     __syncthreads();  // barriers initialised, tensor memory allocated
     asm volatile("tcgen05.fence::after_thread_sync;");
     const uint32_t tmem = *tmem_slot;
+    const int stride = (int)gridDim.x;
 
     if (warp == 0) {
-        // ---- control (one lane): halo copies kHaloBufs tiles ahead, MMA issue
-        int issued_halo = 0, issued_mma = 0;  // tiles of this CTA (in order) whose copies / MMAs were issued
-        if (lane == 0)
-            for (int j = 0; j < kHaloBufs; ++j)
-                if ((int)blockIdx.x + j * (int)gridDim.x < ntiles) {
-                    conv_issue_halo(&tin, halo + j * kHaloBytes, halo_bar + 8 * j, blockIdx.x + j * gridDim.x,
-                                    tiles_x, rows2);
-                    ++issued_halo;
-                }
-        __syncwarp();
+        // ---- control (one lane): MMA issue
         // the whole warp meets the epilogue warps, which staged the weights
         asm volatile("bar.sync 3, %0;" ::"n"(kCtlThreads + kEpiThreads) : "memory");
         if (lane == 0) {
             const uint64_t a_desc0 = umma_desc(smem_addr(sa)), b_desc0 = umma_desc(smem_addr(sb));
             uint32_t it = 0;
-            for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++it) {
+            int issued_mma = 0;  // tiles of this CTA (in order) whose MMAs were issued
+            for (int tile = blockIdx.x; tile < ntiles; tile += stride, ++it) {
                 const int s = it & 1;
-                // A set s written and halo buffer s read by the producers
-                if (!mbar_wait_bounded(afull_bar + 8 * s, (it >> 1) & 1, abort)) {
-                    *abort = 1;
-                    break;
-                }
-                // halo buffer it % kHaloBufs was read by the producers for this tile
-                const int ahead = tile + kHaloBufs * gridDim.x, hb = it % kHaloBufs;
-                if (ahead < ntiles) {
-                    conv_issue_halo(&tin, halo + hb * kHaloBytes, halo_bar + 8 * hb, ahead, tiles_x, rows2);
-                    ++issued_halo;
-                }
-                // accumulator set s drained by the epilogue of tile it-2
-                if (it >= 2 && !mbar_wait_bounded(empty_bar + 8 * s, ((it >> 1) - 1) & 1, abort)) {
+                // A set s written; accumulator set s drained by the epilogue of tile it-2
+                if (!mbar_wait_bounded(afull_bar + 8 * s, (it >> 1) & 1, abort) ||
+                    (it >= 2 && !mbar_wait_bounded(empty_bar + 8 * s, ((it >> 1) - 1) & 1, abort))) {
                     *abort = 1;
                     break;
                 }
@@ -263,12 +329,13 @@ __global__ void __launch_bounds__(kConvThreads, 1)
                 // descriptors differ from the first one only in their start
                 // address field (no carry: shared addresses stay below 256 KB)
                 const uint64_t a_set = a_desc0 + (uint64_t)(s * (kOpASet >> 4));
+                const uint64_t b_set = b_desc0 + (uint64_t)(tile >= n0 ? kOpBConv >> 4 : 0);
 #pragma unroll
                 for (int a = 0; a < 4; ++a)
 #pragma unroll
                     for (int ks = 0; ks < kConvK / 16; ++ks) {
                         const uint64_t ad = a_set + (uint64_t)((a * kOpABytes + ks * 256) >> 4);
-                        const uint64_t bd = b_desc0 + (uint64_t)(((a & 1) * kOpBBytes + ks * 256) >> 4);
+                        const uint64_t bd = b_set + (uint64_t)(((a & 1) * kOpBBytes + ks * 256) >> 4);
                         asm volatile("{\n .reg .pred p;\n setp.ne.u32 p, %4, 0;\n"
                                      " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(
                                          tmem + s * kAccCols + a * kConvN),
@@ -278,35 +345,28 @@ __global__ void __launch_bounds__(kConvThreads, 1)
                     full_bar + 8 * s));
                 ++issued_mma;
             }
-            if (*abort) {
-                // let the copies and MMAs in flight land before the CTA frees
-                // its memory (bounded waits that ignore the abort flag)
+            if (*abort && issued_mma > 0) {
+                // the MMAs in flight finish before the CTA frees tensor memory
+                // (a bounded wait that ignores the abort flag)
                 const volatile int no_abort = 0;
-                // the last copy into buffer j was tile index jl = the largest
-                // index below issued_halo that is j modulo kHaloBufs
-                for (int j = 0; j < kHaloBufs && j < issued_halo; ++j) {
-                    const int jl = j + (issued_halo - 1 - j) / kHaloBufs * kHaloBufs;
-                    mbar_wait_bounded(halo_bar + 8 * j, (jl / kHaloBufs) & 1, &no_abort);
-                }
-                if (issued_mma > 0) {
-                    const int last = issued_mma - 1;
-                    mbar_wait_bounded(full_bar + 8 * (last & 1), (last >> 1) & 1, &no_abort);
-                }
+                const int last = issued_mma - 1;
+                mbar_wait_bounded(full_bar + 8 * (last & 1), (last >> 1) & 1, &no_abort);
             }
         }
         __syncwarp();
     } else if (warp <= kProdThreads / 32) {
-        // ---- producers: row m of the four A operands of every tile
-        const int m = tid - kCtlThreads;
+        // ---- producers, team s: row m of the four A operands of its tiles
+        const int s = (tid - kCtlThreads) / kTeamThreads, m = (tid - kCtlThreads) % kTeamThreads;
         int woff[3];  // byte offsets of halo words m+3, m+4, m+5 (L, C, R), each in its box
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
             const int wq = m + 3 + q, box = wq >= kHaloBox / 2;
             woff[q] = box * kHaloBoxStride + (wq - box * (kHaloBox / 2)) * 4;
         }
-        uint32_t it = 0;
-        for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++it) {
-            const int s = it & 1, hb = it % kHaloBufs;
+        unsigned char *As = sa + s * kOpASet;
+        uint32_t it = s;
+        for (int tile = blockIdx.x + s * stride; tile < ntiles; tile += 2 * stride, it += 2) {
+            const int hb = it % kHaloBufs;
             const bool hok = mbar_wait_bounded(halo_bar + 8 * hb, (it / kHaloBufs) & 1, abort);
             // A set s was last read by the MMAs of tile it-2
             const bool aok = it < 2 || mbar_wait_bounded(full_bar + 8 * s, ((it >> 1) - 1) & 1, abort);
@@ -325,7 +385,6 @@ __global__ void __launch_bounds__(kConvThreads, 1)
                     Cw[ci * 4 + r] = *reinterpret_cast<const uint32_t *>(row + woff[1]);
                     Rw[ci * 4 + r] = *reinterpret_cast<const uint32_t *>(row + woff[2]);
                 }
-            unsigned char *As = sa + s * kOpASet;
 #pragma unroll
             for (int dy = 0; dy < 2; ++dy)
 #pragma unroll
@@ -353,84 +412,69 @@ __global__ void __launch_bounds__(kConvThreads, 1)
                 }
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // generic stores -> tensor-core reads
             __syncwarp();
-            if (lane == 0) mbar_arrive(afull_bar + 8 * s);
+            if (lane == 0) {
+                // every value read from the halo has been written to A above
+                mbar_arrive(afull_bar + 8 * s);
+                mbar_arrive(hempty_bar + 8 * hb);
+            }
         }
-    } else {
-        // ---- epilogue: stage the weights once, then per tile read TMEM lanes
-        // 32*quad.., channels 32*chalf .. +31, pooled column x0/2 + mo
-        const int etid = tid - kCtlThreads - kProdThreads;
-        {
-            // the weights and the bias, raw, into staging buffer 1 (which the
-            // epilogue of tile 1 writes first): one round of independent loads
-            constexpr int kW = kConvN * kConvTaps, kWPer = (kW + kEpiThreads - 1) / kEpiThreads;
-            uint16_t *wraw = reinterpret_cast<uint16_t *>(stage + kStageBytes);
-            float *braw = reinterpret_cast<float *>(stage + kStageBytes + 2 * kW);
-            const unsigned short *wsrc = reinterpret_cast<const unsigned short *>(wt);
-            unsigned short wl[kWPer];
-#pragma unroll
-            for (int r = 0; r < kWPer; ++r) {
-                const int i = etid + r * kEpiThreads;
-                wl[r] = i < kW ? __ldg(wsrc + i) : (unsigned short)0;
+    } else if (warp == kConvThreads / 32 - 1) {
+        // ---- loader (one lane): halo copies kHaloBufs tiles ahead
+        if (lane == 0) {
+            asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&pair.m[0].tin)) : "memory");
+            uint32_t it = 0;
+            for (int tile = blockIdx.x; tile < ntiles; tile += stride, ++it) {
+                const int hb = it % kHaloBufs;
+                if (it >= kHaloBufs && !mbar_wait_bounded(hempty_bar + 8 * hb, ((it / kHaloBufs) - 1) & 1, abort)) {
+                    *abort = 1;
+                    break;
+                }
+                const bool second = tile >= n0;
+                conv_issue_halo(pair.m[second], halo + hb * kHaloBytes, halo_bar + 8 * hb, tile - (second ? n0 : 0));
             }
-            const float bl = etid < kConvN ? __ldg(bias + etid) : 0.f;
-#pragma unroll
-            for (int r = 0; r < kWPer; ++r) {
-                const int i = etid + r * kEpiThreads;
-                if (i < kW) wraw[i] = wl[r];
-            }
-            if (etid < kConvN) braw[etid] = bl;
-            asm volatile("bar.sync 2, %0;" ::"n"(kEpiThreads) : "memory");
-            // the two B operands in the K order from the raw copy, one 16-byte
-            // core-matrix row (eight K positions of one channel) per store.
-            // Thread etid builds the rows of channel etid % 64 at K chunk
-            // etid / 64 (uniform over a warp) for both parities: the chunk
-            // is matched against compile-time values, so every tap index
-            // below is a constant
-            constexpr int kKc = kConvK / 8;
-            static_assert(kEpiThreads == kConvN * kKc, "one channel and K chunk per epilogue thread");
-            const int co = etid % kConvN, kq = etid / kConvN;
-            const float bb = braw[co];
-            const __nv_bfloat16 bhi = __float2bfloat16_rn(bb);
-            const uint32_t bias_hi = __bfloat16_as_ushort(bhi);
-            const uint32_t bias_lo = __bfloat16_as_ushort(__float2bfloat16_rn(bb - __bfloat162float(bhi)));
-#pragma unroll
-            for (int kc = 0; kc < kKc; ++kc) {
-                if (kc != kq) continue;
-#pragma unroll
-                for (int p = 0; p < 2; ++p) {
-                    uint32_t q[4];
-#pragma unroll
-                    for (int j = 0; j < 8; j += 2) {
-                        uint32_t two = 0;
-#pragma unroll
-                        for (int h2 = 0; h2 < 2; ++h2) {
-                            const int k = 8 * kc + j + h2, tap = conv_tap(p, k);
-                            const uint32_t v = tap >= 0 ? (uint32_t)wraw[co * kConvTaps + tap]
-                                                        : (k == 27 ? bias_hi : (k == 28 ? bias_lo : 0u));
-                            two |= v << (16 * h2);
-                        }
-                        q[j / 2] = two;
-                    }
-                    *reinterpret_cast<uint4 *>(sb + p * kOpBBytes + umma_off(co, 8 * kc)) =
-                        make_uint4(q[0], q[1], q[2], q[3]);
+            if (*abort) {
+                // the copies in flight land before the CTA frees its memory
+                // (bounded waits that ignore the abort flag): the last copy
+                // into buffer j was tile index jl, the largest below `it` that
+                // is j modulo kHaloBufs
+                const volatile int no_abort = 0;
+                for (uint32_t j = 0; j < (uint32_t)kHaloBufs && j < it; ++j) {
+                    const uint32_t jl = j + (it - 1 - j) / kHaloBufs * kHaloBufs;
+                    mbar_wait_bounded(halo_bar + 8 * j, (jl / kHaloBufs) & 1, &no_abort);
                 }
             }
+        }
+        __syncwarp();
+    } else {
+        // ---- epilogue: stage the weights once, then team s reads TMEM lanes
+        // 32*quad.. of its tiles' accumulators, pooled column x0/2 + mo
+        const int etid = tid - kCtlThreads - kProdThreads;
+        {
+            // raw copies in the team buffers that are written last (tiles 2 and 3)
+            unsigned char *raw0 = stage + kStageBytes, *raw1 = stage + 3 * kStageBytes;
+            conv_load_raw(pair.m[0], raw0, etid);
+            if (ntiles > n0) conv_load_raw(pair.m[1], raw1, etid);
+            asm volatile("bar.sync 2, %0;" ::"n"(kEpiThreads) : "memory");
+            conv_build_b(raw0, sb, etid);
+            if (ntiles > n0) conv_build_b(raw1, sb + kOpBConv, etid);
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // B: generic stores -> tensor-core reads
             asm volatile("bar.sync 3, %0;" ::"n"(kCtlThreads + kEpiThreads) : "memory");
         }
-        const int ew = warp - (kCtlThreads + kProdThreads) / 32, quad = warp & 3, chalf = ew >> 2;
+        const int s = etid / kTeamThreads, et = etid % kTeamThreads, quad = warp & 3;
         const int mo = quad * 32 + lane;
-        uint32_t it = 0;
-        for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++it) {
-            const int s = it & 1;
+        unsigned char *sg0 = stage + 2 * s * kStageBytes;
+        uint32_t it = s;
+        for (int tile = blockIdx.x + s * stride; tile < ntiles; tile += 2 * stride, it += 2) {
+            const bool second = tile >= n0;
+            const Conv &m = pair.m[second];
             int b, y0, x0;  // the tile's coordinates, computed while its MMAs may still run
-            conv_tile_coords(tile, tiles_x, rows2, b, y0, x0);
+            conv_tile_coords(tile - (second ? n0 : 0), m.tiles_x, m.rows2, b, y0, x0);
             const bool fok = mbar_wait_bounded(full_bar + 8 * s, (it >> 1) & 1, abort);
             asm volatile("tcgen05.fence::after_thread_sync;");
-            unsigned char *sg = stage + s * kStageBytes;
+            unsigned char *sg = sg0 + ((it >> 1) & 1) * kStageBytes;
 #pragma unroll
-            for (int chunk = 0; chunk < 2; ++chunk) {
-                const int c0 = 32 * chalf + 16 * chunk;
+            for (int chunk = 0; chunk < kConvN / 16; ++chunk) {
+                const int c0 = 16 * chunk;
                 uint32_t v[4][16];
 #pragma unroll
                 for (int a = 0; a < 4; ++a) {
@@ -443,7 +487,7 @@ __global__ void __launch_bounds__(kConvThreads, 1)
                         : "r"(taddr));
                 }
                 asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                if (chunk == 1) {
+                if (chunk == kConvN / 16 - 1) {
                     // this warp is done with accumulator set s
                     asm volatile("tcgen05.fence::before_thread_sync;");
                     __syncwarp();
@@ -469,20 +513,20 @@ __global__ void __launch_bounds__(kConvThreads, 1)
                 }
             }
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // staging writes -> TMA store reads
-            // the store of the previous tile must be done reading its staging
-            // buffer before the next tile writes it
-            if (etid == 0 && tma_store) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-            if (!bar_and(2, kEpiThreads, fok && !*abort)) {
-                if (etid == 0) *abort = 1;
+            // the store of the team's previous tile must be done reading its
+            // buffer before the team's next tile writes it
+            if (et == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+            if (!bar_and(4 + s, kTeamThreads, fok && !*abort)) {
+                if (et == 0) *abort = 1;
                 break;
             }
-            if (tma_store) {
+            if (m.tma_store) {
                 // one TMA store of the 128 x 1 x 64 box at (x0/2, y0/2, 64b);
                 // the hardware drops the columns past the image edge
-                if (etid == 0) {
+                if (et == 0) {
                     asm volatile(
                         "cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%1, %2, %3}], [%4];" ::"l"(
-                            reinterpret_cast<uint64_t>(&tout)),
+                            reinterpret_cast<uint64_t>(&m.tout)),
                         "r"(x0 >> 1), "r"(y0 >> 1), "r"(kConvN * b), "r"(smem_addr(sg))
                         : "memory");
                     asm volatile("cp.async.bulk.commit_group;" ::: "memory");
@@ -490,20 +534,23 @@ __global__ void __launch_bounds__(kConvThreads, 1)
             } else {
                 // pooled rows not a multiple of 8 values: 8-byte stores of
                 // whole vectors (the valid width, wo - x0/2 capped at 128, is
-                // a multiple of 4); the next tile writes the other buffer
+                // a multiple of 4); the team's next tile writes the other buffer
+                const int ho = m.h / 2, wo = m.w / 2;
                 const int valid = min(kTileCols / 2, wo - (x0 >> 1));
-                __nv_bfloat16 *orow = out + (((size_t)b * kConvN) * ho + (y0 >> 1)) * wo + (x0 >> 1);
+                __nv_bfloat16 *orow = m.out + (((size_t)b * kConvN) * ho + (y0 >> 1)) * wo + (x0 >> 1);
                 const size_t plane = (size_t)ho * wo;
                 const uint2 *src = reinterpret_cast<const uint2 *>(sg);
-                for (int i = etid; i < kConvN * (kTileCols / 8); i += kEpiThreads) {
+                for (int i = et; i < kConvN * (kTileCols / 8); i += kTeamThreads) {
                     const int ch = i / (kTileCols / 8), j = i % (kTileCols / 8);
                     if (4 * j < valid) *reinterpret_cast<uint2 *>(orow + ch * plane + 4 * j) = src[i];
                 }
             }
         }
-        if (etid == 0 && tma_store) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+        if (et == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
     }
-    if (tid == 0 && *abort) atomicExch(status, 1);
+    if (tid == 0 && *abort)
+        for (int q = 0; q < 2; ++q)
+            if (pair.m[q].ntiles > 0) atomicExch(pair.m[q].status, 1);
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(kTmemCols));
@@ -511,31 +558,48 @@ __global__ void __launch_bounds__(kConvThreads, 1)
 
 // e[p] = mean of plane p (hw bf16 values), fp32 per thread, fixed-order
 // block tree; one block per plane.  128-bit loads when every plane starts on
-// a 16-byte boundary (hw % 8 == 0 and an aligned base), scalar loads
-// otherwise.
-__global__ void __launch_bounds__(256) avgpool_global_kernel(const __nv_bfloat16 *__restrict__ p,
-                                                             float *__restrict__ e, int hw, int vec)
+// a 16-byte boundary (hw % 8 == 0 and an aligned base), eight of a thread in
+// flight, each one's eight values summed as a tree; scalar loads otherwise.
+// A launch does one input, or the two of a merged launch (blocks [0, planes)
+// of the grid the first).
+struct AvgPool {
+    const __nv_bfloat16 *p;
+    float *e;
+    int hw, vec, planes;
+};
+struct AvgPoolPair {
+    AvgPool m[2];
+};
+
+__global__ void __launch_bounds__(256) avgpool_global_kernel(const __grid_constant__ AvgPoolPair pair)
 {
     __shared__ double sh[256 / 32];
+    const bool second = (int)blockIdx.x >= pair.m[0].planes;
+    const AvgPool &m = pair.m[second];
+    const int plane = (int)blockIdx.x - (second ? pair.m[0].planes : 0), hw = m.hw;
     float s = 0.f;
-    if (vec) {
-        const uint4 *q = reinterpret_cast<const uint4 *>(p + (size_t)blockIdx.x * hw);
-#pragma unroll 4
-        for (int i = threadIdx.x; i < hw / 8; i += 256) {
-            const uint4 v = q[i];
-            const uint32_t u[4] = {v.x, v.y, v.z, v.w};
+    if (m.vec) {
+        const uint4 *q = reinterpret_cast<const uint4 *>(m.p + (size_t)plane * hw);
+        constexpr int kV = 8;
+        for (int i = threadIdx.x; i < hw / 8; i += kV * 256) {
+            uint4 v[kV];
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                s += __uint_as_float(u[k] << 16);
-                s += __uint_as_float(u[k] & 0xFFFF0000u);
+            for (int k = 0; k < kV; ++k) v[k] = i + k * 256 < hw / 8 ? __ldg(q + i + k * 256) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+            for (int k = 0; k < kV; ++k) {
+                const uint32_t u[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
+                float t[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) t[j] = __uint_as_float(u[j] << 16) + __uint_as_float(u[j] & 0xFFFF0000u);
+                s += (t[0] + t[1]) + (t[2] + t[3]);
             }
         }
     } else {
-        const __nv_bfloat16 *q = p + (size_t)blockIdx.x * hw;
+        const __nv_bfloat16 *q = m.p + (size_t)plane * hw;
         for (int i = threadIdx.x; i < hw; i += 256) s += __bfloat162float(q[i]);
     }
     const double t = block_sum((double)s, sh);
-    if (threadIdx.x == 0) e[blockIdx.x] = (float)(t / hw);
+    if (threadIdx.x == 0) m.e[plane] = (float)(t / hw);
 }
 
 // out[b][j] = bd[j] + sum_i e1[b][i] wd[i][j] + sum_i e2[b][i] wd[c+i][j]:
@@ -598,57 +662,85 @@ struct ConvMaps {
     CUtensorMap tin, tout;
 };
 
-int launch_conv(const LaunchArgs &a, void *s)
+// The tensor maps of one convolution.  Per process: raise the dynamic
+// shared-memory limit once (no attribute calls on later launches, so the launch
+// can be stream-captured), and keep the tensor maps of the last few (buffer,
+// shape) combinations.
+cudaError_t conv_maps(const LaunchArgs &a, Conv &out)
 {
     const int n = a.i32(5), h = a.i32(6), w = a.i32(7);
     const int wo = w / 2, tma_store = wo % 8 == 0;
-    // per process: raise the dynamic shared-memory limit once (no attribute
-    // calls on later launches, so the launch can be stream-captured), and
-    // keep the tensor maps of the last few (buffer, shape) combinations
     static std::mutex mu;
     static bool configured = false;
     static ConvMaps cache[8];
     static int cache_next = 0;
-    ConvMaps maps;
-    {
-        std::lock_guard<std::mutex> lock(mu);
-        if (!configured) {
-            cudaError_t e = cudaFuncSetAttribute(conv3x3_relu_pool_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 (int)kConvSmem);
-            if (e != cudaSuccess) return e;
-            configured = true;
-        }
-        int hit = -1;
-        for (int i = 0; i < 8; ++i)
-            if (cache[i].x == a.ptr[0] && cache[i].out == a.ptr[3] && cache[i].n == n && cache[i].h == h &&
-                cache[i].w == w)
-                hit = i;
-        if (hit < 0) {
-            ConvMaps m;
-            m.x = a.ptr[0];
-            m.out = a.ptr[3];
-            m.n = n;
-            m.h = h;
-            m.w = w;
-            std::memset(&m.tin, 0, sizeof m.tin);
-            std::memset(&m.tout, 0, sizeof m.tout);
-            if (!encode_bf16_3d(&m.tin, a.ptr[0], (uint64_t)w, (uint64_t)h, (uint64_t)3 * n, kHaloBox, 4, 3))
-                return cudaErrorNotSupported;
-            if (tma_store && !encode_bf16_3d(&m.tout, a.ptr[3], (uint64_t)wo, (uint64_t)(h / 2), (uint64_t)kConvN * n,
-                                             kTileCols / 2, 1, kConvN))
-                return cudaErrorNotSupported;
-            hit = cache_next;
-            cache[hit] = m;
-            cache_next = (cache_next + 1) % 8;
-        }
-        maps = cache[hit];
+    std::lock_guard<std::mutex> lock(mu);
+    if (!configured) {
+        cudaError_t e = cudaFuncSetAttribute(conv3x3_relu_pool_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)kConvSmem);
+        if (e != cudaSuccess) return e;
+        configured = true;
     }
-    const int64_t tiles = (int64_t)n * (h / 2) * ceil_div(w, kTileCols);
+    int hit = -1;
+    for (int i = 0; i < 8; ++i)
+        if (cache[i].x == a.ptr[0] && cache[i].out == a.ptr[3] && cache[i].n == n && cache[i].h == h && cache[i].w == w)
+            hit = i;
+    if (hit < 0) {
+        ConvMaps m;
+        m.x = a.ptr[0];
+        m.out = a.ptr[3];
+        m.n = n;
+        m.h = h;
+        m.w = w;
+        std::memset(&m.tin, 0, sizeof m.tin);
+        std::memset(&m.tout, 0, sizeof m.tout);
+        if (!encode_bf16_3d(&m.tin, a.ptr[0], (uint64_t)w, (uint64_t)h, (uint64_t)3 * n, kHaloBox, 4, 3))
+            return cudaErrorNotSupported;
+        if (tma_store && !encode_bf16_3d(&m.tout, a.ptr[3], (uint64_t)wo, (uint64_t)(h / 2), (uint64_t)kConvN * n,
+                                         kTileCols / 2, 1, kConvN))
+            return cudaErrorNotSupported;
+        hit = cache_next;
+        cache[hit] = m;
+        cache_next = (cache_next + 1) % 8;
+    }
+    out.tin = cache[hit].tin;
+    out.tout = cache[hit].tout;
+    return cudaSuccess;
+}
+
+// One convolution, or the two of a merged launch.
+int launch_conv_run(const LaunchArgs *const *m, int count, void *s)
+{
+    ConvPair pair;
+    std::memset(&pair, 0, sizeof pair);
+    int64_t tiles = 0;
+    for (int i = 0; i < count; ++i) {
+        const LaunchArgs &a = *m[i];
+        const int n = a.i32(5), h = a.i32(6), w = a.i32(7);
+        Conv &c = pair.m[i];
+        const cudaError_t e = conv_maps(a, c);
+        if (e != cudaSuccess) return e;
+        c.wt = a.p<__nv_bfloat16>(1);
+        c.bias = a.p<float>(2);
+        c.out = a.p<__nv_bfloat16>(3);
+        c.status = a.p<int>(4);
+        c.h = h;
+        c.w = w;
+        c.tma_store = (w / 2) % 8 == 0;
+        c.tiles_x = (int)ceil_div(w, kTileCols);
+        c.rows2 = h / 2;
+        c.ntiles = n * c.rows2 * c.tiles_x;
+        tiles += c.ntiles;
+    }
     const unsigned grid = (unsigned)(tiles < sm_count() ? tiles : sm_count());
-    conv3x3_relu_pool_kernel<<<grid, kConvThreads, kConvSmem, (cudaStream_t)s>>>(
-        maps.tin, maps.tout, a.p<__nv_bfloat16>(1), a.p<float>(2), a.p<__nv_bfloat16>(3), a.p<int>(4), n, h, w,
-        tma_store);
+    conv3x3_relu_pool_kernel<<<grid, kConvThreads, kConvSmem, (cudaStream_t)s>>>(pair);
     return cudaGetLastError();
+}
+
+int launch_conv(const LaunchArgs &a, void *s)
+{
+    const LaunchArgs *m[1] = {&a};
+    return launch_conv_run(m, 1, s);
 }
 
 const char *validate_avgpool(const LaunchArgs &a)
@@ -660,13 +752,54 @@ const char *validate_avgpool(const LaunchArgs &a)
     return nullptr;
 }
 
+int launch_avgpool_run(const LaunchArgs *const *m, int count, void *s)
+{
+    AvgPoolPair pair = {};
+    int blocks = 0;
+    for (int i = 0; i < count; ++i) {
+        const LaunchArgs &a = *m[i];
+        const int hw = a.i32(3);
+        pair.m[i] = AvgPool{a.p<__nv_bfloat16>(0), a.p<float>(1), hw,
+                            hw % 8 == 0 && (reinterpret_cast<uintptr_t>(a.ptr[0]) & 15) == 0, a.i32(2)};
+        blocks += pair.m[i].planes;
+    }
+    avgpool_global_kernel<<<(unsigned)blocks, 256, 0, (cudaStream_t)s>>>(pair);
+    return cudaGetLastError();
+}
+
 int launch_avgpool(const LaunchArgs &a, void *s)
 {
-    const int hw = a.i32(3);
-    const int vec = hw % 8 == 0 && (reinterpret_cast<uintptr_t>(a.ptr[0]) & 15) == 0;
-    avgpool_global_kernel<<<(unsigned)a.i32(2), 256, 0, (cudaStream_t)s>>>(a.p<__nv_bfloat16>(0), a.p<float>(1), hw,
-                                                                           vec);
-    return cudaGetLastError();
+    const LaunchArgs *m[1] = {&a};
+    return launch_avgpool_run(m, 1, s);
+}
+
+// The same kernel on two inputs, the two branches of the DL program: the next
+// launch of it that shares nothing written with the first.  One grid pays one
+// start-up and one part-filled last round (4096 tiles over 152 CTAs make 27
+// rounds, 2048 make 14), and the host one launch.
+template <MergeLaunchFn LAUNCH> bool merge_branches(const RunLaunch *run, int n, Merge &out)
+{
+    const RunLaunch &f = run[0];
+    // work items (tiles or planes), which one grid counts in 32 bits
+    auto items = [](const LaunchArgs &a) {
+        return a.nargs == 8 ? (int64_t)a.i32(5) * (a.i32(6) / 2) * ceil_div(a.i32(7), kTileCols) : (int64_t)a.i32(2);
+    };
+    for (int j = 1; j < n; ++j) {
+        const RunLaunch &g = run[j];
+        if (g.k != f.k) continue;
+        bool apart = items(f.a) + items(g.a) <= INT32_MAX / 2;
+        for (int p = 0; p < f.a.nargs; ++p)
+            for (int q = 0; q < g.a.nargs; ++q)
+                if (f.array[p] >= 0 && f.array[p] == g.array[q])
+                    apart = apart && f.k->spec[p].mode == GDAG_MODE_IN && g.k->spec[q].mode == GDAG_MODE_IN;
+        if (!apart) return false;
+        out.count = 2;
+        out.member[0] = 0;
+        out.member[1] = j;
+        out.launch = LAUNCH;
+        return true;
+    }
+    return false;
 }
 
 const char *validate_dense(const LaunchArgs &a)
@@ -711,8 +844,10 @@ void append_dl_kernels(std::vector<KernelEntry> &v)
                       {arr(GDAG_MODE_IN), arr(GDAG_MODE_IN), arr(GDAG_MODE_IN), arr(GDAG_MODE_OUT),
                        arr(GDAG_MODE_INOUT), scal(4), scal(4), scal(4)},
                       validate_conv, launch_conv));
+    v.back().merge = merge_branches<launch_conv_run>;
     v.push_back(entry("avgpool_global", (const void *)avgpool_global_kernel,
                       {arr(GDAG_MODE_IN), arr(GDAG_MODE_OUT), scal(4), scal(4)}, validate_avgpool, launch_avgpool));
+    v.back().merge = merge_branches<launch_avgpool_run>;
     v.push_back(entry("concat_dense", (const void *)concat_dense_kernel,
                       {arr(GDAG_MODE_IN), arr(GDAG_MODE_IN), arr(GDAG_MODE_IN), arr(GDAG_MODE_IN), arr(GDAG_MODE_OUT),
                        scal(4), scal(4), scal(4)},

@@ -225,3 +225,103 @@ def test_ml_program_equals_its_launches():
             got.append([t.clone() for t in (m.S1, m.S2, m.labels)])
     for a, b in zip(*got):
         assert torch.equal(a, b)
+
+
+# one tile in all; more tiles than SMs in either; odd counts, so that a CTA's
+# two teams end on different convolutions; a plain-store row width (w / 2 not a
+# multiple of 8) beside a tensor-store one, both ways round; a partial tile
+@pytest.mark.parametrize("a,b", [((1, 2, 8), (1, 2, 8)), ((1, 2, 64), (1, 4, 264)), ((1, 4, 264), (2, 6, 72)),
+                                 ((2, 6, 72), (3, 66, 192)), ((5, 130, 128), (1, 2, 520)), ((3, 110, 256), (4, 90, 256))])
+def test_two_convolutions_and_pools_equal_their_launches(a, b):
+    g = np.random.default_rng(sum(a) * 31 + sum(b))
+    bf = torch.bfloat16
+    ins = []
+    for n, h, w in (a, b):
+        ins.append((torch.from_numpy(g.random((n, 3, h, w), dtype=np.float32)).to(bf),
+                    torch.from_numpy(g.normal(0, 0.3, (64, 3, 3, 3)).astype(np.float32)).to(bf),
+                    torch.from_numpy(g.normal(0, 0.1, 64).astype(np.float32))))
+    got = []
+    for policy, want in ((G.GDAG_POLICY_PARALLEL, 2), (G.GDAG_POLICY_SERIAL_ASYNC, 4)):
+        with G.Context(policy=policy) as ctx:
+            p, outs, keep = ctx.program(), [], []
+            pools = []
+            for (n, h, w), (x, wt, bias) in zip((a, b), ins):
+                t = [v.cuda() for v in (x, wt, bias)]
+                o = torch.full((n, 64, h // 2, w // 2), -1.0, dtype=bf, device="cuda")
+                e = torch.full((n, 64), -1.0, device="cuda")
+                st = torch.zeros(1, dtype=torch.int32, device="cuda")
+                A = [ctx.array(v) for v in t + [o, st, e]]
+                p.launch("conv3x3_relu_pool", A[0], A[1], A[2], A[3], A[4], n, h, w)
+                pools.append((A[3], A[5], n * 64, (h // 2) * (w // 2)))
+                outs += [o, e, st]
+                keep += t + A
+            for q in pools:
+                p.launch("avgpool_global", *q)
+            torch.cuda.synchronize()
+            for _ in range(2):
+                assert launches(ctx, p.issue) == want
+            got.append([t.clone() for t in outs])
+    for x, y in zip(*got):
+        assert torch.equal(x.view(torch.int16) if x.dtype == bf else x, y.view(torch.int16) if y.dtype == bf else y)
+    assert got[0][2].item() == 0 and got[0][5].item() == 0
+    # the first convolution against plain float64
+    (n, h, w), (x, wt, bias) = a, ins[0]
+    ref = torch.nn.functional.conv2d(x.double(), wt.double(), bias.double(), padding=1).clamp_min(0)
+    ref = torch.nn.functional.max_pool2d(ref, 2)
+    assert (got[0][0].double().cpu() - ref).abs().max() <= 2.0 ** -8 * ref.abs().max()
+
+
+# sizes that merge; one pair whose lengths differ; the empty vector
+@pytest.mark.parametrize("n,nnz,m,mnz", [(1, 0, 1, 0), (500, 4000, 500, 4000), (3000, 0, 100, 9000), (1279, 1, 1281, 7),
+                                         (60_000, 300_000, 20_000, 500_000), (0, 0, 50, 60)])
+def test_two_products_norms_and_scalings_equal_their_launches(n, nnz, m, mnz):
+    got = []
+    for policy, want in ((G.GDAG_POLICY_PARALLEL, 3), (G.GDAG_POLICY_SERIAL_ASYNC, 6)):
+        with G.Context(policy=policy) as ctx:
+            p, outs, keep, tail = ctx.program(), [], [], []
+            for k, (rows, nz) in enumerate(((n, nnz), (m, mnz))):
+                g = np.random.default_rng(rows + nz)
+                ends = np.sort(g.integers(0, rows + 1, nz)) if rows else np.zeros(0, np.int64)
+                if rows and nz > 100:  # a row that spans many tiles
+                    ends[nz // 4: 3 * nz // 4] = ends[nz // 2]
+                rp = np.searchsorted(ends, np.arange(rows + 1), side="left").astype(np.int32)
+                rp[-1] = nz if rows else 0
+                col = g.integers(0, max(rows, 1), max(nz, 1)).astype(np.int32)
+                val = g.normal(0, 1, max(nz, 1)).astype(np.float32)
+                x = g.normal(0, 1, max(rows, 1)).astype(np.float32)
+                t = [torch.from_numpy(v).cuda() for v in (rp, col, val, x)]
+                y = torch.full((max(rows, 1),), 7.0, device="cuda")
+                nrm = torch.full((1,), -1.0, device="cuda")
+                sc = [torch.zeros(G.gdag_scratch_bytes(q, rows + nz), dtype=torch.uint8, device="cuda")
+                      for q in ("spmv_partition", "spmv_csr", "l2norm")]
+                A = [ctx.array(v) for v in t + [y, nrm] + sc]
+                ctx.launch("spmv_partition", A[0], A[6], rows, nz)
+                p.launch("spmv_csr", A[0], A[1], A[2], A[3], A[6], A[4], A[7], rows, nz)
+                tail.append((A[4], A[5], A[8], rows))
+                outs += [y, nrm]
+                keep += t + sc + A
+                if k == 0 and policy == G.GDAG_POLICY_PARALLEL and rows:
+                    ref = np.zeros(rows)
+                    np.add.at(ref, np.searchsorted(rp[1:], np.arange(nz), side="right"),
+                              val[:nz].astype(np.float64) * x[col[:nz]])
+                    mag = np.zeros(rows)
+                    np.add.at(mag, np.searchsorted(rp[1:], np.arange(nz), side="right"),
+                              np.abs(val[:nz].astype(np.float64) * x[col[:nz]]))
+            for v, q, s, rows in tail:
+                p.launch("l2norm", v, q, s, rows)
+            for v, q, s, rows in tail:
+                p.launch("scale", v, q, rows)
+            ctx.sync()
+            k = launches(ctx, p.issue)
+            assert k == want
+            got.append([t.clone() for t in outs])
+    for a, b in zip(*got):
+        assert same_bits(a, b)
+    if n:
+        y, nrm = got[0][0].double().cpu().numpy()[:n], got[0][1].item()
+        assert abs(nrm - np.sqrt((ref ** 2).sum())) <= 1e-5 * max(nrm, 1e-30) + 1e-30
+        # a product rounds once, a sum of up to 64 terms in a chain, the rest in
+        # trees and per tile, the norm and the division once each: under 256 ulp
+        # halves of the sum of |terms|
+        if nrm > 0:
+            assert (np.abs(y * nrm - ref) <= 2.0 ** -24 * 256 * mag + 1e-30).all()

@@ -292,3 +292,47 @@ def test_score_and_softmax_programs():
         assert n == want, (kw, n)
         ctx.close()
         one.close()
+
+
+def test_branch_programs():
+    """Two launches of one kernel on separate data merge; ones that share what
+    either writes do not, nor larger ones than a rule takes."""
+    at = itertools.count(1)
+
+    def case(make, want):
+        ctx = G.Context(backend="fake", record_log=True)
+        seq = make(lambda nb: ctx.array(dev=next(at) << 34, nbytes=nb))
+        nodes, n = issue(ctx, seq)
+        assert n == want, (seq[0][0], n)
+        ctx.close()
+
+    sb = G.gdag_scratch_bytes
+
+    def spmv(arr, n, nnz, same_carry=False):
+        rp, col, val, x = arr(4 * (n + 1)), arr(4 * nnz), arr(4 * nnz), arr(4 * n)
+        part, c = arr(sb("spmv_partition", n + nnz)), arr(sb("spmv_csr", n + nnz))
+        c2 = c if same_carry else arr(sb("spmv_csr", n + nnz))
+        return [("spmv_csr", rp, col, val, x, part, arr(4 * n), q, n, nnz) for q in (c, c2)]
+    case(lambda a: spmv(a, 1000, 5000), 1)                   # one matrix, two results
+    case(lambda a: spmv(a, 1000, 5000, same_carry=True), 2)
+    case(lambda a: spmv(a, 700_000, 3_600_000), 2)           # over 2^22 rows and nonzeros
+    case(lambda a: [("scale", a(4000), a(4), 1000), ("scale", a(8000), a(4), 2000)], 1)
+    case(lambda a: [("scale", a(8 << 20), a(4), 1 << 21), ("scale", a(4000), a(4), 1000)], 2)
+
+    def shared_norm(a):
+        x = a(4000)
+        return [("scale", x, a(4), 1000), ("scale", a(4000), x, 1000)]
+    case(shared_norm, 2)
+
+    def chain(a):  # the second product reads the first's result
+        s = spmv(a, 1000, 5000)
+        return [s[0], s[1][:4] + (s[0][6],) + s[1][5:]]
+    case(chain, 2)
+
+    def conv(a, same_status=False):
+        x, w, b, st = a(2 * 3 * 64 * 64), a(2 * 64 * 27), a(256), a(4)
+        return [("conv3x3_relu_pool", x, w, b, a(2 * 64 * 32 * 32), q, 1, 64, 64)
+                for q in (st, st if same_status else a(4))]
+    case(conv, 1)
+    case(lambda a: conv(a, True), 2)
+    case(lambda a: [("avgpool_global", a(2 * 64 * 100), a(256), 64, 100), ("avgpool_global", a(2 * 64 * 100), a(256), 64, 100)], 1)
