@@ -8,6 +8,9 @@
 #include "backend.h"
 
 namespace gdag {
+
+cudaError_t host_copy(void *dst, const void *src, size_t bytes, const void *host, cudaStream_t s, bool *done);  // host_copy.cu
+
 namespace {
 
 // Sticky errors leave the CUDA context unusable; everything else is local to
@@ -128,10 +131,16 @@ class CudaBackend final : public Backend {
     }
     int copy_h2d(void *dst, const void *src, size_t bytes, void *s) override
     {
+        bool done;
+        const int r = chk(host_copy(dst, src, bytes, src, (cudaStream_t)s, &done), "host-to-device copy kernel");
+        if (r || done) return r;
         return chk(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, (cudaStream_t)s), "cudaMemcpyAsync H2D");
     }
     int copy_d2h(void *dst, const void *src, size_t bytes, void *s) override
     {
+        bool done;
+        const int r = chk(host_copy(dst, src, bytes, dst, (cudaStream_t)s, &done), "device-to-host copy kernel");
+        if (r || done) return r;
         return chk(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, (cudaStream_t)s), "cudaMemcpyAsync D2H");
     }
     int external(void (*fn)(void *, void *), void *user, void *s) override
