@@ -130,8 +130,9 @@ struct Ctx {
     std::vector<gdag_op> op_log;
     gdag_stats st{};
 
-    // scratch for one element
-    std::vector<int64_t> par;
+    // scratch for one element or one call
+    std::vector<int64_t> par, retire_stack, ext;
+    std::vector<uint8_t> issued_early;
 
     // stream capture (CUDA graphs of a repeated DAG shape)
     bool capturing = false;
@@ -257,7 +258,8 @@ struct Ctx {
     // complete once the host has observed id's completion).
     void retire(int64_t id)
     {
-        std::vector<int64_t> stack{id};
+        std::vector<int64_t> &stack = retire_stack;
+        stack.assign(1, id);
         while (!stack.empty()) {
             int64_t v = stack.back();
             stack.pop_back();
@@ -485,10 +487,34 @@ struct Ctx {
         return GDAG_OK;
     }
 
-    // Optionally retire completed parents without a host wait.
+    // Whether the element goes on a parent's stream (pick_stream's first rule)
+    // with every active parent there: then it waits for nothing, and whether the
+    // parents are complete changes nothing for it.
+    bool follows_parents() const
+    {
+        if (opt.policy != GDAG_POLICY_PARALLEL) return false;
+        int32_t s = -1;
+        bool first = false;
+        for (int64_t p : par) {
+            if (p < base) continue;
+            const Node &n = nodes[(size_t)(p - base)];
+            if (!n.active) continue;
+            if (n.stream < 0 || (s >= 0 && n.stream != s)) return false;
+            s = n.stream;
+            first = first || (streams[(size_t)s].tail == p && !n.first_child_taken);
+        }
+        return first;
+    }
+
+    // Optionally retire completed parents without a host wait.  A query costs
+    // the host about 2 us, as much as a launch, so an element that follows its
+    // parents on their stream asks only once kAskAt elements are active (they
+    // are retired with their ancestors, a whole chain at a time).
+    static constexpr int64_t kAskAt = 64;
     int retire_done_parents()
     {
         if (!opt.retire_by_query || capturing) return GDAG_OK;
+        if (active_count < kAskAt && follows_parents()) return GDAG_OK;
         // the members of a merged launch share one event: it is asked once
         int32_t pending = -1, ready = -1;
         for (int64_t p : par) {
@@ -1336,13 +1362,12 @@ static bool run_launch(gdag_ctx *c, const gdag_elem &e, const gdag_arg *args, in
         if (a[i].kind == GDAG_ARG_ARRAY && a[i].mode != GDAG_MODE_SIGNATURE && a[i].mode != k.spec[i].mode) return false;
         if (a[i].kind == GDAG_ARG_ARRAY) out.array[i] = a[i].array;
     }
-    const std::string msg = c->last_error;
-    if (resolve(c, e.kernel, e.grid, e.block, 0, a, e.nargs, out.a, acc, nacc)) {
-        c->last_error = msg;
-        return false;
-    }
+    std::string kept;
+    kept.swap(c->last_error);
+    const bool ok = resolve(c, e.kernel, e.grid, e.block, 0, a, e.nargs, out.a, acc, nacc) == GDAG_OK;
+    kept.swap(c->last_error);
     out.k = &k;
-    return true;
+    return ok;
 }
 
 static bool conflicting(const Access *a, int na, const Access *b, int nb)
@@ -1386,21 +1411,26 @@ static bool merge_legal(gdag_ctx *c, MergeRun &q)
     // what a member writes shares no memory with any other array of the unit
     // (other handles may name the same memory: the members would no longer
     // run one after another on it)
+    struct Span {
+        int32_t array;
+        bool written;
+        uintptr_t lo, hi;
+    } span[gdag::kMaxRun * gdag::kMaxArgs];
+    int ns = 0;
     for (int k = 0; k < m.count; ++k)
-        for (int x = 0; x < q.nacc[m.member[k]]; ++x) {
-            const Access &w = q.acc[m.member[k]][x];
-            if (!(w.bits & gdag::W_BIT)) continue;
-            const ArrayState &ws = c->arrays[(size_t)w.array];
-            const uintptr_t w0 = (uintptr_t)ws.dev, w1 = w0 + ws.bytes;
-            for (int l = 0; l < m.count; ++l)
-                for (int y = 0; y < q.nacc[m.member[l]]; ++y) {
-                    const int32_t o = q.acc[m.member[l]][y].array;
-                    if (o == w.array) continue;
-                    const ArrayState &os = c->arrays[(size_t)o];
-                    const uintptr_t o0 = (uintptr_t)os.dev, o1 = o0 + os.bytes;
-                    if (w0 < o1 && o0 < w1) return false;
-                }
+        for (int x = 0, mem = q.order[k]; x < q.nacc[mem]; ++x) {
+            const Access &w = q.acc[mem][x];
+            int i = 0;
+            while (i < ns && span[i].array != w.array) ++i;
+            if (i == ns) {
+                const ArrayState &st = c->arrays[(size_t)w.array];
+                span[ns++] = Span{w.array, false, (uintptr_t)st.dev, (uintptr_t)st.dev + st.bytes};
+            }
+            span[i].written = span[i].written || (w.bits & gdag::W_BIT);
         }
+    for (int i = 0; i < ns; ++i)
+        for (int j = i + 1; j < ns; ++j)
+            if ((span[i].written || span[j].written) && span[i].lo < span[j].hi && span[j].lo < span[i].hi) return false;
     return true;
 }
 
@@ -1414,7 +1444,8 @@ static int issue_merged(gdag_ctx *c, const MergeRun &q, const gdag_elem *elems, 
     const gdag::Merge &m = q.m;
     const int64_t first = c->next_id();
     const LaunchArgs *la[gdag::kMaxRun];
-    std::vector<int64_t> ext;  // active parents outside the unit
+    std::vector<int64_t> &ext = c->ext;  // active parents outside the unit
+    ext.clear();
     for (int k = 0; k < m.count; ++k) {
         const int x = q.order[k];
         la[k] = &q.run[m.member[k]].a;
@@ -1481,7 +1512,8 @@ static int issue_each(gdag_ctx *c, const gdag_elem *elems, int32_t n, const gdag
     if (nodes_out)
         for (int32_t i = 0; i < n; ++i) nodes_out[i] = -1;
     const bool merging = c->opt.policy == GDAG_POLICY_PARALLEL && !c->opt.trace && !c->poisoned;
-    std::vector<uint8_t> done;  // elements issued as members of an earlier unit
+    std::vector<uint8_t> &done = c->issued_early;  // elements issued as members of an earlier unit
+    done.clear();
     for (int32_t i = 0; i < n; ++i) {
         const gdag_elem &e = elems[i];
         if (!done.empty() && done[(size_t)i]) {

@@ -171,6 +171,7 @@ SIGNATURES = {
 
 _lib = None
 _LAUNCH = [None]  # gdag_launch, bound once by lib()
+_ISSUE = [None]   # gdag_issue, likewise
 
 
 class GdagError(RuntimeError):
@@ -192,6 +193,7 @@ def lib():
             f.restype = res
             f.argtypes = args
         _LAUNCH[0] = L.gdag_launch
+        _ISSUE[0] = L.gdag_issue
         _lib = L
     return _lib
 
@@ -879,7 +881,12 @@ class Program:
         plan = {name: [(ew if w == "e" else aw, size, np.asarray(ix, dtype=np.intp))
                        for (w, size), ix in g.items()] for name, g in groups.items()}
         nodes = (_i64 * max(1, n))()
-        self._ready = (elems, args, plan, nodes, _i32(), n, self._nargs)
+        issued = _i32()
+        # the call's arguments, marshalled once (the structures stay alive with
+        # them in the tuple)
+        call = (_vp(ctypes.addressof(elems)), _i32(n), _vp(ctypes.addressof(args)), _i64(self._nargs),
+                _vp(ctypes.addressof(nodes)), ctypes.byref(issued))
+        self._ready = (call, plan, nodes, issued, n, elems, args)
 
     def params(self):
         return sorted({p[0] for p in self._arg_params} | {p[0] for p in self._elem_params})
@@ -891,16 +898,16 @@ class Program:
         and ``nodes``."""
         if self._ready is None:
             self._prepare()
-        elems, args, plan, nodes, issued, n, nargs = self._ready
-        if len(values) != len(plan) or any(k not in values for k in plan):
-            raise GdagError(GDAG_ERR_INVALID, "program parameters %s, given %s"
-                            % (sorted(plan), sorted(values)))
-        for name, targets in plan.items():
-            v = values[name]
-            for words, size, ix in targets:
-                words[ix] = _scalar_bits(v, size)
-        r = lib().gdag_issue(self.ctx.h, ctypes.addressof(elems), n, ctypes.addressof(args), nargs,
-                             ctypes.addressof(nodes), ctypes.byref(issued))
+        call, plan, nodes, issued, n, _, _ = self._ready
+        if plan or values:
+            if len(values) != len(plan) or any(k not in values for k in plan):
+                raise GdagError(GDAG_ERR_INVALID, "program parameters %s, given %s"
+                                % (sorted(plan), sorted(values)))
+            for name, targets in plan.items():
+                v = values[name]
+                for words, size, ix in targets:
+                    words[ix] = _scalar_bits(v, size)
+        r = _ISSUE[0](self.ctx.h, *call)
         out = nodes[:n]
         if r < 0:
             e = GdagError(r, self.ctx.last_error)
