@@ -325,3 +325,42 @@ def test_two_products_norms_and_scalings_equal_their_launches(n, nnz, m, mnz):
         # halves of the sum of |terms|
         if nrm > 0:
             assert (np.abs(y * nrm - ref) <= 2.0 ** -24 * 256 * mag + 1e-30).all()
+
+
+# one plane row; images whose planes take the pools' scalar loads; more tiles and
+# planes than the chip holds at a time
+@pytest.mark.parametrize("n,h,w,classes,swap", [(1, 2, 8, 1, False), (3, 6, 24, 33, True), (2, 66, 264, 10, False),
+                                                (40, 128, 256, 10, True)])
+def test_dl_program_equals_its_launches(n, h, w, classes, swap):
+    g = np.random.default_rng(n * h + w)
+    bf = torch.bfloat16
+    f = lambda *s: torch.from_numpy(g.normal(0, 0.3, s).astype(np.float32))  # noqa: E731
+    ins = [(f(n, 3, h, w).to(bf), f(64, 3, 3, 3).to(bf), f(64)) for _ in range(2)]
+    wd, bd = f(128, classes), f(classes)
+    got = []
+    for policy, want in ((G.GDAG_POLICY_PARALLEL, 1), (G.GDAG_POLICY_SERIAL_ASYNC, 5)):
+        with G.Context(policy=policy) as ctx:
+            x = [[t.cuda() for t in b] for b in ins]
+            P = [torch.zeros((n, 64, h // 2, w // 2), dtype=bf, device="cuda") for _ in x]
+            E = [torch.zeros((n, 64), device="cuda") for _ in x]
+            st = [torch.zeros(1, dtype=torch.int32, device="cuda") for _ in x]
+            dense = [wd.cuda(), bd.cuda(), torch.zeros((n, classes), device="cuda")]
+            AX = [[ctx.array(t) for t in b] for b in x]
+            AP, AE, AS, AD = ([ctx.array(t) for t in v] for v in (P, E, st, dense))
+            p = ctx.program()
+            for k in (0, 1):
+                p.launch("conv3x3_relu_pool", *AX[k], AP[k], AS[k], n, h, w)
+            for k in (1, 0) if swap else (0, 1):
+                p.launch("avgpool_global", AP[k], AE[k], n * 64, (h // 2) * (w // 2))
+            p.launch("concat_dense", AE[0], AE[1], *AD, n, 64, classes)
+            out = []
+            torch.cuda.synchronize()
+            for step in range(3):  # other inputs each time: a stage that ran ahead would show
+                assert launches(ctx, p.issue) == want
+                out += [t.clone() for t in P + E + st + dense[2:]]
+                for b in x:
+                    b[0].mul_(-0.5)
+                torch.cuda.synchronize()
+            got.append(out)
+    for a, b in zip(*got):
+        assert torch.equal(a.view(torch.int16) if a.dtype == bf else a, b.view(torch.int16) if b.dtype == bf else b)

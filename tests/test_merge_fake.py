@@ -336,3 +336,19 @@ def test_branch_programs():
     case(conv, 1)
     case(lambda a: conv(a, True), 2)
     case(lambda a: [("avgpool_global", a(2 * 64 * 100), a(256), 64, 100), ("avgpool_global", a(2 * 64 * 100), a(256), 64, 100)], 1)
+
+    # the convolutions, their pools and the dense layer in a row, and what is not that
+    def dl(a, pools=(0, 1), embed=(0, 1), to=None, between=False):
+        P, E = [a(2 * 64 * 32 * 32) for _ in range(2)], [a(256) for _ in range(2)]
+        seq = [("conv3x3_relu_pool", a(2 * 3 * 64 * 64), a(2 * 64 * 27), a(256), P[k], a(4), 1, 64, 64) for k in range(2)]
+        seq += [("avgpool_global", P[k], E[to[i] if to else k], 64, 1024) for i, k in enumerate(pools)]
+        if between:
+            seq.insert(3, ("scale", a(4000), a(4), 1000))
+        return seq + [("concat_dense", E[embed[0]], E[embed[1]], a(4 * 128 * 10), a(40), a(40), 1, 64, 10)]
+    case(dl, 1)
+    case(lambda a: dl(a, pools=(1, 0)), 1)
+    case(lambda a: dl(a, embed=(1, 0)), 1)
+    case(lambda a: dl(a, pools=(0, 0), to=(0, 1)), 3)        # both pools of one output: the two pairs
+    case(lambda a: dl(a, to=(0, 0)), 4)                      # one embedding written twice
+    case(lambda a: dl(a, embed=(0, 0)), 3)
+    case(lambda a: dl(a, between=True), 4)                   # not in a row: the two pairs and the rest
