@@ -587,7 +587,7 @@ __global__ void __launch_bounds__(256) avgpool_global_kernel(const __grid_consta
         for (int i = threadIdx.x; i < hw / 8; i += kV * 256) {
             uint4 v[kV];
 #pragma unroll
-            for (int k = 0; k < kV; ++k) v[k] = i + k * 256 < hw / 8 ? __ldg(q + i + k * 256) : make_uint4(0u, 0u, 0u, 0u);
+            for (int k = 0; k < kV; ++k) v[k] = i + k * 256 < hw / 8 ? load_dep(q + i + k * 256) : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
             for (int k = 0; k < kV; ++k) {
                 const uint32_t u[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
@@ -598,8 +598,8 @@ __global__ void __launch_bounds__(256) avgpool_global_kernel(const __grid_consta
             }
         }
     } else {
-        const __nv_bfloat16 *q = m.p + (size_t)plane * hw;
-        for (int i = threadIdx.x; i < hw; i += 256) s += __bfloat162float(q[i]);
+        const uint16_t *q = reinterpret_cast<const uint16_t *>(m.p) + (size_t)plane * hw;
+        for (int i = threadIdx.x; i < hw; i += 256) s += __uint_as_float((uint32_t)load_dep(q + i) << 16);
     }
     const double t = block_sum((double)s, sh);
     if (threadIdx.x == 0) m.e[plane] = (float)(t / hw);
@@ -608,7 +608,7 @@ __global__ void __launch_bounds__(256) avgpool_global_kernel(const __grid_consta
 // out[b][j] = bd[j] + sum_i e1[b][i] wd[i][j] + sum_i e2[b][i] wd[c+i][j]:
 // one block per image, one warp per class (strided), the 2c products of a
 // logit split over the lanes and summed by a fixed shuffle tree.
-__global__ void __launch_bounds__(256) concat_dense_kernel(const float *__restrict__ e1, const float *__restrict__ e2,
+__global__ void __launch_bounds__(256) concat_dense_kernel(const float *e1, const float *e2,
                                                            const float *__restrict__ wd, const float *__restrict__ bd,
                                                            float *__restrict__ out, int c, int classes)
 {
@@ -617,7 +617,7 @@ __global__ void __launch_bounds__(256) concat_dense_kernel(const float *__restri
     for (int j = warp; j < classes; j += 256 / 32) {
         float s = 0.f;
         for (int i = lane; i < 2 * c; i += 32) {
-            const float e = i < c ? e1[(size_t)b * c + i] : e2[(size_t)b * c + (i - c)];
+            const float e = load_dep(i < c ? e1 + (size_t)b * c + i : e2 + (size_t)b * c + (i - c));
             s = fmaf(e, wd[(size_t)i * classes + j], s);
         }
 #pragma unroll

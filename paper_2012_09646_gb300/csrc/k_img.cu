@@ -236,7 +236,7 @@ __global__ void __launch_bounds__(kMmThreads) minmax_kernel(const float *__restr
     }
 }
 
-__global__ void __launch_bounds__(kMmCombineThreads) minmax_combine_kernel(const float2 *__restrict__ part,
+__global__ void __launch_bounds__(kMmCombineThreads) minmax_combine_kernel(const float2 *part,
                                                                            float *__restrict__ mm, int blocks)
 {
     __shared__ float smin[kMmCombineThreads / 32], smax[kMmCombineThreads / 32];
@@ -244,7 +244,7 @@ __global__ void __launch_bounds__(kMmCombineThreads) minmax_combine_kernel(const
     asm volatile("griddepcontrol.wait;" ::: "memory");
     float lo = INFINITY, hi = -INFINITY;
     for (int b = threadIdx.x; b < blocks; b += kMmCombineThreads) {
-        const float2 p = part[b];
+        const float2 p = load_dep(part + b);
         lo = fminf(lo, p.x);
         hi = fmaxf(hi, p.y);
     }

@@ -206,12 +206,12 @@ __device__ __forceinline__ void copy4_row(float4 *dst, const float *__restrict__
     }
 }
 
-__device__ __forceinline__ float4 load4_row(const float *__restrict__ in, int rows, int cols, bool vec, int y, int x)
+__device__ __forceinline__ float4 load4_row(const float *in, int rows, int cols, bool vec, int y, int x)
 {
     const float *row = in + (size_t)clampi(y, 0, rows - 1) * cols;
-    if (vec) return __ldg(reinterpret_cast<const float4 *>(row + clampi(x, 0, cols - 4)));
-    return make_float4(__ldg(row + clampi(x, 0, cols - 1)), __ldg(row + clampi(x + 1, 0, cols - 1)),
-                       __ldg(row + clampi(x + 2, 0, cols - 1)), __ldg(row + clampi(x + 3, 0, cols - 1)));
+    if (vec) return load_dep(reinterpret_cast<const float4 *>(row + clampi(x, 0, cols - 4)));
+    return make_float4(load_dep(row + clampi(x, 0, cols - 1)), load_dep(row + clampi(x + 1, 0, cols - 1)),
+                       load_dep(row + clampi(x + 2, 0, cols - 1)), load_dep(row + clampi(x + 3, 0, cols - 1)));
 }
 
 // The vertical sums (lo, hi) of a lane outside the image, which moved whole
@@ -429,8 +429,8 @@ struct Stretch {
 
 template <bool VEC>
 __global__ void __launch_bounds__(kStThreads)
-    img_stage2_kernel(const float *__restrict__ ba, const float *__restrict__ bb, const float *__restrict__ sh,
-                      const float2 *__restrict__ part_a, const float2 *__restrict__ part_b, int pairs,
+    img_stage2_kernel(const float *ba, const float *bb, const float *sh, const float2 *part_a, const float2 *part_b,
+                      int pairs,
                       float *__restrict__ mm_a, float *__restrict__ mm_b, float *__restrict__ ea,
                       float *__restrict__ eb, float *__restrict__ out, int rows, int cols, int th)
 {
@@ -445,7 +445,7 @@ __global__ void __launch_bounds__(kStThreads)
     asm volatile("griddepcontrol.wait;" ::: "memory");
     Range ra, rb;
     for (int b = threadIdx.x; b < pairs; b += kStThreads) {
-        const float2 pa = __ldg(part_a + b), pb = __ldg(part_b + b);
+        const float2 pa = load_dep(part_a + b), pb = load_dep(part_b + b);
         ra.lo = fminf(ra.lo, pa.x);
         ra.hi = fmaxf(ra.hi, pa.y);
         rb.lo = fminf(rb.lo, pb.x);

@@ -81,7 +81,41 @@ template <int Width> constexpr size_t reduce_scratch_bytes()
 // resident while that kernel runs (once every block of it has executed
 // griddepcontrol.launch_dependents) and must execute griddepcontrol.wait,
 // which returns when that kernel has completed and its writes are visible,
-// before it reads anything that kernel wrote.
+// before it reads anything that kernel wrote, and read that by load_dep: the
+// two kernels overlap, so the data is not read-only for this one's lifetime as
+// __ldg and const __restrict__ promise, and such a load may be moved up past the wait
+// (a volatile one is not).
+__device__ __forceinline__ float load_dep(const float *p)
+{
+    float v;
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float2 load_dep(const float2 *p)
+{
+    float2 v;
+    asm volatile("ld.global.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float4 load_dep(const float4 *p)
+{
+    float4 v;
+    asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ uint4 load_dep(const uint4 *p)
+{
+    uint4 v;
+    asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ uint16_t load_dep(const uint16_t *p)
+{
+    uint16_t v;
+    asm volatile("ld.global.u16 %0, [%1];" : "=h"(v) : "l"(p));
+    return v;
+}
+
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_dependent(void (*kernel)(KArgs...), dim3 grid, int threads, cudaStream_t s, Args... args)
 {
