@@ -33,8 +33,10 @@ constexpr int kMlFeatStep = 8;   // features per lane per load (32 bytes)
 // one step fall into different banks.
 __host__ __device__ constexpr int ml_quarter_stride(int feats, int nc4) { return (feats / kMlQuarters) * nc4 * 4 + 4; }
 
-// One launch's table and result, or two launches' over the same X (blockIdx.y
-// picks one).
+// Two launches' tables and results over the same X (blockIdx.y picks one). A single
+// launch keeps plain pointer parameters: read through this structure they lost
+// what __restrict__ says of them, and 100000 x 480 x 16, two launches and their
+// softmaxes, took 118.7 us instead of 114.0.
 struct ScoreTables {
     const float *T[2], *bias[2];
     float *S[2];
@@ -42,12 +44,9 @@ struct ScoreTables {
 };
 
 template <int NC4>
-__global__ void __launch_bounds__(kMlThreads) dense_scores_kernel(const int *__restrict__ X, ScoreTables tb, int rows,
-                                                                  int feats)
+__device__ __forceinline__ void dense_scores_body(const int *__restrict__ X, const float *__restrict__ T, const float *__restrict__ bias,
+                                                   float *__restrict__ S, int rows, int feats, int classes)
 {
-    const float *__restrict__ T = blockIdx.y ? tb.T[1] : tb.T[0], *__restrict__ bias = blockIdx.y ? tb.bias[1] : tb.bias[0];
-    float *__restrict__ S = blockIdx.y ? tb.S[1] : tb.S[0];
-    const int classes = blockIdx.y ? tb.classes[1] : tb.classes[0];
     extern __shared__ float4 smem4[];
     float *st = reinterpret_cast<float *>(smem4);
     const int fq = feats / kMlQuarters;  // features per quarter
@@ -141,6 +140,21 @@ __global__ void __launch_bounds__(kMlThreads) dense_scores_kernel(const int *__r
     }
 }
 
+template <int NC4>
+__global__ void __launch_bounds__(kMlThreads)
+    dense_scores_kernel(const int *__restrict__ X, const float *__restrict__ T, const float *__restrict__ bias,
+              float *__restrict__ S, int rows, int feats, int classes)
+{
+    dense_scores_body<NC4>(X, T, bias, S, rows, feats, classes);
+}
+template <int NC4>
+__global__ void __launch_bounds__(kMlThreads)
+    dense_scores_pair_kernel(const int *__restrict__ X, const __grid_constant__ ScoreTables tb, int rows, int feats)
+{
+    const int k = blockIdx.y;
+    dense_scores_body<NC4>(X, tb.T[k], tb.bias[k], tb.S[k], rows, feats, tb.classes[k]);
+}
+
 // ---- pipelined form (tables that leave room for a staging ring): X is
 // staged in shared memory in slices of kPipeSlice features x kPipeRows rows
 // by cp.async, kPipeStages slices in flight per CTA, so the loads no longer
@@ -175,12 +189,9 @@ __device__ __forceinline__ void cp_async16(void *dst, const void *src, int src_b
 }
 
 template <int NC4>
-__global__ void __launch_bounds__(kPipeThreads, 2)
-    dense_scores_pipe_kernel(const int *__restrict__ X, ScoreTables tb, int rows, int feats)
+__device__ __forceinline__ void dense_scores_pipe_body(const int *__restrict__ X, const float *__restrict__ T, const float *__restrict__ bias,
+                                                   float *__restrict__ S, int rows, int feats, int classes)
 {
-    const float *__restrict__ T = blockIdx.y ? tb.T[1] : tb.T[0], *__restrict__ bias = blockIdx.y ? tb.bias[1] : tb.bias[0];
-    float *__restrict__ S = blockIdx.y ? tb.S[1] : tb.S[0];
-    const int classes = blockIdx.y ? tb.classes[1] : tb.classes[0];
     extern __shared__ float4 smem4[];
     unsigned char *xs = reinterpret_cast<unsigned char *>(smem4);
     float *st = reinterpret_cast<float *>(xs + kPipeStages * kPipeStageBytes);
@@ -303,6 +314,21 @@ __global__ void __launch_bounds__(kPipeThreads, 2)
         }
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
+}
+
+template <int NC4>
+__global__ void __launch_bounds__(kPipeThreads, 2)
+    dense_scores_pipe_kernel(const int *__restrict__ X, const float *__restrict__ T, const float *__restrict__ bias,
+              float *__restrict__ S, int rows, int feats, int classes)
+{
+    dense_scores_pipe_body<NC4>(X, T, bias, S, rows, feats, classes);
+}
+template <int NC4>
+__global__ void __launch_bounds__(kPipeThreads, 2)
+    dense_scores_pipe_pair_kernel(const int *__restrict__ X, const __grid_constant__ ScoreTables tb, int rows, int feats)
+{
+    const int k = blockIdx.y;
+    dense_scores_pipe_body<NC4>(X, tb.T[k], tb.bias[k], tb.S[k], rows, feats, tb.classes[k]);
 }
 
 // v := softmax of v[0 .. classes), max-subtracted.
@@ -447,9 +473,10 @@ template <int NC4> int scores_pipe_launch(const LaunchArgs *const *m, int count,
     const int rows = a.i32(4), feats = a.i32(5), classes = a.i32(6);
     static bool configured = false;
     if (!configured) {
-        cudaError_t e = cudaFuncSetAttribute(dense_scores_pipe_kernel<NC4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             110 * 1024);
-        if (e != cudaSuccess) return e;
+        for (const void *f : {(const void *)dense_scores_pipe_kernel<NC4>, (const void *)dense_scores_pipe_pair_kernel<NC4>}) {
+            const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, 110 * 1024);
+            if (e != cudaSuccess) return e;
+        }
         configured = true;
     }
     // an equal number of tiles for every CTA (to within one): waves of two
@@ -457,8 +484,13 @@ template <int NC4> int scores_pipe_launch(const LaunchArgs *const *m, int count,
     const int64_t ntiles = ceil_div(rows, kPipeRows), slots = 2 * (int64_t)sm_count();
     const int64_t per = ceil_div(ntiles, slots);
     const int64_t grid = ceil_div(ntiles, per);
-    dense_scores_pipe_kernel<NC4><<<dim3((unsigned)grid, (unsigned)count), kPipeThreads, pipe_smem(feats, classes), s>>>(
-        a.p<int>(0), score_tables(m, count), rows, feats);
+    const size_t smem = pipe_smem(feats, classes);
+    if (count == 2)
+        dense_scores_pipe_pair_kernel<NC4><<<dim3((unsigned)grid, 2), kPipeThreads, smem, s>>>(
+            a.p<int>(0), score_tables(m, count), rows, feats);
+    else
+        dense_scores_pipe_kernel<NC4><<<(unsigned)grid, kPipeThreads, smem, s>>>(a.p<int>(0), a.p<float>(1), a.p<float>(2),
+                                                                               a.p<float>(3), rows, feats, classes);
     return cudaGetLastError();
 }
 
@@ -476,9 +508,10 @@ template <int NC4> int scores_launch(const LaunchArgs *const *m, int count, cuda
     static size_t occ_smem = 0;
     static int occ_blocks = 0;
     if (!configured) {
-        cudaError_t e = cudaFuncSetAttribute(dense_scores_kernel<NC4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             200 * 1024);
-        if (e != cudaSuccess) return e;
+        for (const void *f : {(const void *)dense_scores_kernel<NC4>, (const void *)dense_scores_pair_kernel<NC4>}) {
+            const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+            if (e != cudaSuccess) return e;
+        }
         configured = true;
     }
     if (occ_smem != smem) {
@@ -492,8 +525,12 @@ template <int NC4> int scores_launch(const LaunchArgs *const *m, int count, cuda
     const int64_t groups = ceil_div(rows, 16 * (kMlThreads / 32));
     int64_t grid = (int64_t)sm_count() * per_sm;
     if (grid > groups) grid = groups;
-    dense_scores_kernel<NC4><<<dim3((unsigned)grid, (unsigned)count), kMlThreads, smem, s>>>(
-        a.p<int>(0), score_tables(m, count), rows, feats);
+    if (count == 2)
+        dense_scores_pair_kernel<NC4><<<dim3((unsigned)grid, 2), kMlThreads, smem, s>>>(a.p<int>(0), score_tables(m, count),
+                                                                                      rows, feats);
+    else
+        dense_scores_kernel<NC4><<<(unsigned)grid, kMlThreads, smem, s>>>(a.p<int>(0), a.p<float>(1), a.p<float>(2),
+                                                                          a.p<float>(3), rows, feats, classes);
     return cudaGetLastError();
 }
 
@@ -614,12 +651,21 @@ KernelEntry entry(const char *name, const void *fn, std::initializer_list<gdag_a
 
 }  // namespace
 
-// Both tables padded to the same width: the two halves of one grid.  X comes
-// from L2 for the second; what is saved is a launch, which bounds the small
-// shapes that these forms mostly see.
-MergeLaunchFn scores_cuda_pair(int feats, int classes0, int classes1)
+// Both tables padded to the same width: the two halves of one grid. What it saves is a
+// launch, an event and a second stream, which bound a short step; a long one loses
+// the overlap of two grids, the second half's blocks following the first's. The line
+// is the work of one table. Two launches on two streams against the pair, three
+// programs in turn, us a step: below it 16000 x 96 x 8 (3.1e6) 16.1 and 7.7, 24000 x
+// 352 x 2 (8.4e6) 15.9 and 10.1, 50000 x 96 x 8 (9.6e6) 20.9 and 20.4; above it
+// 28000 x 96 x 16 (1.1e7) 17.1 and 17.6, 32768 x 480 x 2 (1.6e7) 17.0 and 19.4,
+// 100000 x 480 x 16 (1.9e8) 114.0 and 120.0.
+constexpr int64_t kPairWork = 10000000;
+
+MergeLaunchFn scores_cuda_pair(int rows, int feats, int classes0, int classes1)
 {
-    return nc4_of(classes0) == nc4_of(classes1) && use_pipe(feats, classes0) == use_pipe(feats, classes1)
+    const int nc4 = nc4_of(classes0);
+    return nc4 == nc4_of(classes1) && use_pipe(feats, classes0) == use_pipe(feats, classes1) &&
+                   (int64_t)rows * feats * nc4 <= kPairWork
                ? launch_scores_cuda
                : nullptr;
 }

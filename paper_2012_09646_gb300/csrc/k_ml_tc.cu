@@ -610,7 +610,7 @@ int launch_scores_tc(const LaunchArgs &a, cudaStream_t s)
 // What launches the two dense_scores launches f and g (which share X, rows and
 // feats) as one: on the tensor cores, reading X once; on the CUDA cores, the
 // halves of one grid; nullptr where the two take different forms.
-MergeLaunchFn scores_cuda_pair(int feats, int classes0, int classes1);
+MergeLaunchFn scores_cuda_pair(int rows, int feats, int classes0, int classes1);
 
 // Two dense_scores launches over the same X (the two classifiers of the ML
 // program).
@@ -626,7 +626,7 @@ bool merge_scores(const RunLaunch *run, int n, Merge &out)
         const bool t0 = scores_tc_ok(feats, c0), t1 = scores_tc_ok(feats, c1);
         MergeLaunchFn launch = nullptr;
         if (t0 && t1 && c0 <= ScPair::kPer && c1 <= ScPair::kPer) launch = launch_scores_pair;
-        else if (!t0 && !t1) launch = scores_cuda_pair(feats, c0, c1);
+        else if (!t0 && !t1) launch = scores_cuda_pair(f.a.i32(4), feats, c0, c1);
         if (!launch) continue;
         // the two results are apart, and no input is a result
         const int32_t s0 = f.array[3], s1 = g.array[3];

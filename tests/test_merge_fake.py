@@ -352,3 +352,20 @@ def test_branch_programs():
     case(lambda a: dl(a, to=(0, 0)), 4)                      # one embedding written twice
     case(lambda a: dl(a, embed=(0, 0)), 3)
     case(lambda a: dl(a, between=True), 4)                   # not in a row: the two pairs and the rest
+
+
+@pytest.mark.parametrize("rows,feats,classes,want", [
+    (52083, 96, 8, 4),      # 9 999 936 products of one table's padded width: the halves of one grid
+    (52084, 96, 8, 5),      # just above: two launches
+    (20000, 480, 4, 2), (20000, 480, 5, 3),  # the padded width counts
+    (100000, 96, 1, 4), (100000, 1024, 10, 4),  # the tensor-core pair has no such line
+])
+def test_cuda_core_score_pairs_end_at_their_line(rows, feats, classes, want):
+    ctx = G.Context(backend="fake", record_log=True)
+    at = itertools.count(1)
+    arr = lambda nb: ctx.array(dev=next(at) << 33, nbytes=nb)  # noqa: E731
+    X, S = arr(4 * rows * feats), [arr(4 * rows * classes) for _ in range(2)]
+    seq = [("dense_scores", X, arr(4 * feats * classes), arr(4 * classes), s, rows, feats, classes) for s in S]
+    seq += [("row_softmax", s, rows, classes) for s in S] + [("argmax_combine", *S, arr(4 * rows), rows, classes)]
+    assert issue(ctx, seq)[1] == want
+    ctx.close()
