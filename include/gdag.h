@@ -466,11 +466,11 @@ int gdag_launch_external(gdag_ctx *ctx, void (*fn)(void *stream, void *user),
  * short DAGs (the comparison with CUDA Graphs, Section IV-D, finds the
  * runtime's overhead negligible only for computations longer than a few
  * milliseconds).  gdag_issue takes several consecutive
- * non-blocking elements of a program in one call; element i is inferred,
- * placed and issued exactly as its own call would be (gdag_launch,
- * gdag_launch_fused, gdag_array_write with src NULL, or
- * gdag_array_prefetch_host), in order, so the DAG, the streams, the waits
- * and the results are those of the single calls.
+ * non-blocking elements of a program in one call; element i is what its own
+ * call would make it (gdag_launch, gdag_launch_fused, gdag_array_write with
+ * src NULL, or gdag_array_prefetch_host), in order, so the DAG and the
+ * results are those of the single calls. So are the streams and waits, but
+ * for the merged launches below.
  *
  * Merged launches: under the PARALLEL policy, with trace = 0, consecutive
  * launches of built-in kernels (automatic shape, the signature's access
@@ -486,12 +486,15 @@ int gdag_launch_external(gdag_ctx *ctx, void (*fn)(void *stream, void *user),
  * The units:
  *   vec_square x 2, vec_reduce_diff of the same two arrays;
  *   independent bs_call launches of up to 2^21 options each;
- *   dense_scores x 2 over the same X, rows and feats (up to 10 classes each, or
- *     any of the CUDA-core shapes);
+ *   dense_scores x 2 over the same X, rows and feats (up to 10 classes each on the
+ *     tensor cores; on the CUDA cores one padded width, up to 1e7 products of
+ *     rows, feats and that width over four);
  *   row_softmax x 2, argmax_combine of the same two matrices, up to 32768 rows;
  *   two independent launches of spmv_csr (up to 2^22 rows and nonzeros each), or
  *     of l2norm, scale, seg_l2norm or seg_scale (up to 2^20 elements each);
  *   two independent launches of conv3x3_relu_pool or of avgpool_global;
+ *   conv3x3_relu_pool x 2, avgpool_global of their outputs and concat_dense of
+ *     these, in a row;
  *   gauss_blur x 2, sobel x 2, minmax x 2, extend x 2, unsharp, combine (the
  *     IMG program, the second blur the wider one, radii up to 4).           */
 #define GDAG_ELEM_LAUNCH        0  /* gdag_launch                            */

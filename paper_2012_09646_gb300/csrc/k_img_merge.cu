@@ -11,7 +11,7 @@
 //            each edge map again in its stretched form, and writes e1, e2 and
 //            out.
 // Measured at 4096 x 4096, steps one after another: 113 us a step, from 220 us as
-// ten launches (0.88 of the measured HBM rate for the unit's 671 MB); 12.5 us
+// ten launches (0.88 of the measured HBM rate for the unit's 671 MB); 9 us
 // from 46 us at 512 x 512, where ten launches cost the host 4 us each; 38 us from
 // 53 us at 1300 x 3001, whose rows allow no 128-bit access.
 // Computing Sobel twice costs arithmetic that both stages have to spare (they

@@ -781,8 +781,9 @@ class Program:
     """A recorded sequence of non-blocking elements of a program -- kernel
     launches, fused launches, host writes from the array's host view, and
     prefetches to the host -- issued by ONE gdag_issue call.  This is
-    argument marshalling only: the library infers, places and issues each
-    element exactly as its single call would.  Scalars may be :class:`Param`
+    argument marshalling only: the library infers each element as its single
+    call would, and issues launches that a merged kernel can do together as one
+    unit.  Scalars may be :class:`Param`
     objects whose values are bound at each :meth:`issue`, so one recording
     serves every size of a request shape; the arrays are fixed at recording.
     """

@@ -9,9 +9,10 @@ streams, events and copies are entirely the library's.
 
 With ``batched=True`` (the default) the non-blocking elements of a step are
 recorded once as a :class:`~paper_2012_09646_gb300.gdag.Program` and issued
-with one ``gdag_issue`` call per step; the library infers, places and
-issues each element exactly as one call per element would (``batched=False``),
-but the host's per-element cost leaves the critical path of short DAGs.
+with one ``gdag_issue`` call per step; the library infers each element as one
+call per element would (``batched=False``) and gives the same results, but the
+host's per-element cost leaves the critical path of short DAGs, and launches
+that a merged kernel can do together are issued as one unit.
 """
 from __future__ import annotations
 
