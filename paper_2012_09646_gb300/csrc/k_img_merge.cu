@@ -243,8 +243,9 @@ __global__ void __launch_bounds__(kStThreads, 4)
     const int x = blockIdx.x * kMgCols + 4 * (lane - kMgHL);
     const int y0 = (blockIdx.y * kStWarps + warp) * th;  // th is even
     const bool stores = lane >= kMgHL && lane < 32 - kMgHL && x < cols;
-    // warps of the first and last strips see the image's left or right edge
-    const bool edge = blockIdx.x == 0 || (int)(blockIdx.x + 1) * kMgCols + 4 > cols;
+    // warps of the first and last strips see the image's left or right edge: lane 31
+    // holds columns (blockIdx.x + 1) * kMgCols + 4 .. + 7, and lane 30's blur reads them
+    const bool edge = blockIdx.x == 0 || (int)(blockIdx.x + 1) * kMgCols + 8 > cols;
     Range ra, rb;
     if (y0 < rows) {  // the whole warp
         const int yend = min(y0 + th, rows);

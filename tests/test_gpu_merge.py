@@ -55,6 +55,28 @@ def test_img_program_equals_its_launches(rows, cols, special):
         if fine.any() else True
 
 
+# widths around the last columns that a strip's halo lanes hold (112 k + 4 and 112 k
+# + 8): the edge maps' largest steps lie beside the left or the right edge, so a
+# column taken wrongly there moves the range and with it e5, e9 and out
+@pytest.mark.parametrize("cols", [224, 225, 227, 228, 229, 231, 232, 340, 344, 452, 1012, 4036])
+@pytest.mark.parametrize("columns", [(-4, -1), (-1, None), (-8, -4), (1, 4), (0, 1), (4, 8)])
+def test_img_range_beside_the_edges(cols, columns):
+    rows = 8
+    img = np.zeros((rows, cols), np.float32)
+    img[:, slice(*columns)] = 1.0
+    got = []
+    for policy in (G.GDAG_POLICY_PARALLEL, G.GDAG_POLICY_SERIAL_ASYNC):
+        with G.Context(policy=policy) as ctx:
+            d = ImgDag(ctx, rows, cols)
+            d.img.copy_(torch.from_numpy(img.reshape(-1)))
+            torch.cuda.synchronize()
+            d.launch_all()
+            ctx.sync()
+            got.append([t.clone() for t in (d.b5, d.b9, d.s, d.mm5, d.mm9, d.e5, d.e9)])
+    for a, b in zip(*got):
+        assert same_bits(a, b)
+
+
 @pytest.mark.parametrize("ra,rb,merged", [(1, 2, True), (1, 3, True), (1, 4, True), (2, 3, True), (3, 4, True),
                                           (2, 2, False), (4, 2, False), (2, 5, False)])
 def test_img_program_radii(ra, rb, merged):
