@@ -389,14 +389,15 @@ __global__ void __launch_bounds__(kScThreads, 1)
             // release must not rest on the order of the loads alone, with a wait
             // between them and their first use.
             const bool wide = __any_sync(0xffffffffu, vrange > 2u * kScXmax);
-            if (lane == 0) {
-                if (wide) bad[it & 3] = it;
-                mbar_arrive(xempty + 8 * xsl);
-            }
+            if (lane == 0) mbar_arrive(xempty + 8 * xsl);
             if (!__all_sync(0xffffffffu, step < kASt || mbar_wait_bounded(aempty + 8 * st, ((step / kASt) - 1) & 1, abort))) {
                 if (lane == 0) *abort = 1;
                 break;
             }
+            // Only now: the stage kASt back has been multiplied, so tile it - 2 or a
+            // later one has its accumulators, which the epilogue gave up after it had
+            // read the flag of tile it - 4, whose slot this is.
+            if (wide && lane == 0) bad[it & 3] = it;
             unsigned char *A = sa + st * L::kABytes;
 #pragma unroll
             for (int j = 0; j < kJ; ++j)
@@ -473,11 +474,13 @@ __global__ void __launch_bounds__(kScThreads, 1)
             }
             asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
             asm volatile("tcgen05.fence::before_thread_sync;");
+            // before the accumulators are given up: after that the producers may reach
+            // tile it + 4, whose flag has the same slot
+            const bool wide = bad[it & 3] == it;
             __syncwarp();
             if (lane == 0) mbar_arrive(accempty + 8 * s);
             const int row = tile * kScM + r;
             if (row < rows) {
-                const bool wide = bad[it & 3] == it;
 #pragma unroll
                 for (int t = 0; t < L::kTables; ++t) {
                     const int classes = tb.classes[t];

@@ -92,6 +92,35 @@ def test_scores_out_of_bf16_range_rows_fall_back_exactly(classes):
     ctx.close()
 
 
+# tiles of one, two and three stages, five or more a CTA: a tile's range flag must
+# outlast the epilogue's slow rows of the tile before it.  Values that bfloat16 does
+# not hold in every tile, and in every other group of tiles.  With one flag lost a
+# whole tile would be scored from rounded values, off by up to 2^-9 of its terms
+@pytest.mark.parametrize("feats,classes", [(64, 10), (64, 16), (128, 10), (128, 16), (192, 10)])
+@pytest.mark.parametrize("every", [True, False])
+@pytest.mark.parametrize("policy", [G.GDAG_POLICY_PARALLEL, G.GDAG_POLICY_SERIAL_ASYNC])
+def test_scores_wide_values_in_many_tiles(feats, classes, every, policy):
+    rows = 100_000
+    g = np.random.default_rng(feats + classes)
+    X = g.integers(-1000, 1001, (rows, feats)).astype(np.int32)
+    if not every:
+        X[(np.arange(rows) // 128) % 3 != 0] //= 4
+    T1, T2 = (g.normal(0, 1, (feats, classes)).astype(np.float32) for _ in range(2))
+    b1, b2 = (g.normal(0, 1, classes).astype(np.float32) for _ in range(2))
+    ref = [(N.scores(X, T, b), TOL * np.maximum(N.scores_abs(X, T, b), 1.0)) for T, b in ((T1, b1), (T2, b2))]
+    with G.Context(policy=policy) as ctx:
+        d = MlDag(ctx, rows, feats, classes)
+        d.load(X, T1, b1, T2, b2)
+        p = ctx.program()
+        for T, b, S in ((d.T1A, d.b1A, d.S1A), (d.T2A, d.b2A, d.S2A)):
+            p.launch("dense_scores", d.XA, T, b, S, rows, feats, classes)
+        for _ in range(5):
+            p.issue()
+            ctx.sync()
+            for (want, tol), S in zip(ref, (d.S1, d.S2)):
+                assert np.all(np.abs(S[:rows].cpu().numpy() - want) <= tol)
+
+
 def test_scores_full_size_bit_exact():
     """The benchmark's shape, 100000 x 1024 x 10 (782 tiles over the
     persistent grid, a 32-row last tile): every score bit-exact."""
