@@ -190,3 +190,37 @@ def test_hits_full_size_properties():
         want = N.spmv_csr(sub_rp, sub_col, sub_val, a1) / nh
         got = h2[rows]
         assert np.all(np.abs(got - want) <= 2 * TOL * np.maximum(np.abs(want), 1e-30))
+
+
+def chains_of_seven(p, phase):
+    """float32 row sums of p (rows x k): chains of at most seven products, the
+    first one cut by `phase`, then a tree."""
+    parts, q, n = [], 0, 7 - phase
+    while q < p.shape[1]:
+        s = np.zeros(len(p), np.float32)
+        for j in range(q, min(q + n, p.shape[1])):
+            s = s + p[:, j]
+        parts.append(s)
+        q, n = q + n, 7
+    while len(parts) > 1:
+        parts = [sum(parts[i + 1:i + 2], parts[i]) for i in range(0, len(parts), 2)]
+    return parts[0]
+
+
+# a thread's rows (with 0 to 3 products past the groups of four) and a warp's: as
+# near to 64 bits as short chains and a tree.  40000 rows fix a root mean square to
+# about 0.4%; the factor 1.1 leaves room for the rows that tiles cut
+@pytest.mark.parametrize("k", [4, 5, 7, 16, 24, 31, 40, 48, 51, 56, 63, 64, 65, 200])
+def test_spmv_error_of_row_sums(k):
+    rows = 40_000
+    g = np.random.default_rng(k)
+    x = g.random(rows).astype(np.float32)
+    col = g.integers(0, rows, (rows, k)).astype(np.int32)
+    rowptr = np.arange(rows + 1, dtype=np.int64) * k
+    p = x[col]
+    ref = p.astype(np.float64).sum(1)
+    rms = lambda s: np.sqrt((((s - ref) / ref) ** 2).mean())  # noqa: E731
+    with G.Context() as ctx:
+        got = rms(spmv_gpu(ctx, rowptr, col.reshape(-1), np.ones(rows * k), x))
+    chains = np.sqrt(np.mean([rms(chains_of_seven(p, q)) ** 2 for q in range(7)]))
+    assert got <= 1.1 * chains, (got, chains)
