@@ -659,8 +659,9 @@ struct Ctx {
         return GDAG_OK;
     }
 
-    // The node's work was issued but its event was not recorded, so no
-    // later element could wait for it.  The host waits for its stream
+    // The node's work was issued, in whole or (a launch of several kernels of
+    // which a later one was refused) in part, but its event was not recorded, so
+    // no later element could wait for it.  The host waits for its stream
     // instead (the work and, through the stream's waits, the node's
     // parents) and retires it; if that wait fails too, only the node is
     // retired.  The error `rc` and its message are kept.
@@ -1058,7 +1059,7 @@ int gdag_launch(gdag_ctx *c, gdag_kernel k, gdag_dim3 grid, gdag_dim3 block, siz
     c->log_op(GDAG_OP_LAUNCH, s, -1, id);
     ++c->st.launches;
     r = c->be->launch(c->kernels[(size_t)k], la, c->streams[(size_t)s].handle);
-    if (r) return c->abort_node(id, r, "launch");
+    if (r) return c->unrecorded(id, s, c->be_fail(r, "launch"));
     return c->finish(id, s);
 }
 
@@ -1123,7 +1124,7 @@ int gdag_launch_fused(gdag_ctx *c, gdag_kernel k, const gdag_arg *args, int32_t 
     ++c->st.launches;
     c->st.fused_members += count;
     r = c->be->launch_fused(c->kernels[(size_t)k], la.data(), count, c->streams[(size_t)s].handle);
-    if (r) return c->abort_node(id, r, "fused launch");
+    if (r) return c->unrecorded(id, s, c->be_fail(r, "fused launch"));
     return c->finish(id, s);
 }
 
@@ -1469,7 +1470,7 @@ static int issue_merged(gdag_ctx *c, const MergeRun &q, const gdag_elem *elems, 
         const std::string msg = c->last_error;
         bool done = true;
         if (!c->capturing && !c->poisoned) {
-            if (stream >= 0) {  // launched but not recorded: wait for its stream
+            if (stream >= 0) {  // launched, in part or without a record: wait for its stream
                 c->log_op(GDAG_OP_STREAM_SYNC, stream, -1, -1);
                 ++c->st.host_waits;
                 done = c->poll_stream(stream) == GDAG_OK;
@@ -1492,7 +1493,7 @@ static int issue_merged(gdag_ctx *c, const MergeRun &q, const gdag_elem *elems, 
     c->log_op(GDAG_OP_LAUNCH, s, -1, last);
     ++c->st.launches;
     r = c->be->launch_merged(m, la, q.run[0].k->name.c_str(), c->streams[(size_t)s].handle);
-    if (r) return drop(c->be_fail(r, "merged launch"), -1);
+    if (r) return drop(c->be_fail(r, "merged launch"), s);  // some of its kernels may be running
     r = c->record_end(last, s);
     if (r) return drop(r, s);
     const int32_t slot = c->node(last)->event;

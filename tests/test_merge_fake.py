@@ -369,3 +369,21 @@ def test_cuda_core_score_pairs_end_at_their_line(rows, feats, classes, want):
     seq += [("row_softmax", s, rows, classes) for s in S] + [("argmax_combine", *S, arr(4 * rows), rows, classes)]
     assert issue(ctx, seq)[1] == want
     ctx.close()
+
+
+@pytest.mark.parametrize("merged", [True, False])
+def test_a_launch_that_fails_is_waited_for_on_its_stream(merged):
+    """A launch of several kernels may fail after its first ones run: its stream is
+    synchronised before the elements are retired and the stream is offered again."""
+    ctx = G.Context(backend="fake", fake_fail_op=0, record_log=True)
+    g = Img(ctx)
+    with pytest.raises(G.GdagError) as e:
+        if merged:
+            issue(ctx, g.launches())
+        else:
+            ctx.launch(*g.launches()[4])
+    assert e.value.code == G.GDAG_ERR_CUDA
+    ops = [(o[0], o[1]) for o in ctx.ops()]
+    assert ops == [(G.GDAG_OP_LAUNCH, 0), (G.GDAG_OP_STREAM_SYNC, 0)]
+    assert ctx.stats()["active"] == 0
+    ctx.close()
