@@ -9,7 +9,8 @@
 
 namespace gdag {
 
-cudaError_t host_copy(void *dst, const void *src, size_t bytes, const void *host, cudaStream_t s, bool *done);  // host_copy.cu
+// host_copy.cu
+cudaError_t host_copy(void *dst, const void *src, size_t bytes, const void *host, bool beside, cudaStream_t s, bool *done);
 
 namespace {
 
@@ -129,17 +130,17 @@ class CudaBackend final : public Backend {
         if (e == cudaSuccess) e = cudaGetLastError();
         return chk(e, name);
     }
-    int copy_h2d(void *dst, const void *src, size_t bytes, void *s) override
+    int copy_h2d(void *dst, const void *src, size_t bytes, bool beside, void *s) override
     {
         bool done;
-        const int r = chk(host_copy(dst, src, bytes, src, (cudaStream_t)s, &done), "host-to-device copy kernel");
+        const int r = chk(host_copy(dst, src, bytes, src, beside, (cudaStream_t)s, &done), "host-to-device copy kernel");
         if (r || done) return r;
         return chk(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, (cudaStream_t)s), "cudaMemcpyAsync H2D");
     }
-    int copy_d2h(void *dst, const void *src, size_t bytes, void *s) override
+    int copy_d2h(void *dst, const void *src, size_t bytes, bool beside, void *s) override
     {
         bool done;
-        const int r = chk(host_copy(dst, src, bytes, dst, (cudaStream_t)s, &done), "device-to-host copy kernel");
+        const int r = chk(host_copy(dst, src, bytes, dst, beside, (cudaStream_t)s, &done), "device-to-host copy kernel");
         if (r || done) return r;
         return chk(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, (cudaStream_t)s), "cudaMemcpyAsync D2H");
     }
@@ -220,8 +221,8 @@ class FakeBackend final : public Backend {
     int launch(const KernelEntry &, const LaunchArgs &, void *) override { return op(); }
     int launch_fused(const KernelEntry &, const LaunchArgs *, int, void *) override { return op(); }
     int launch_merged(const Merge &, const LaunchArgs *const *, const char *, void *) override { return op(); }
-    int copy_h2d(void *, const void *, size_t, void *) override { return op(); }
-    int copy_d2h(void *, const void *, size_t, void *) override { return op(); }
+    int copy_h2d(void *, const void *, size_t, bool, void *) override { return op(); }
+    int copy_d2h(void *, const void *, size_t, bool, void *) override { return op(); }
     int external(void (*fn)(void *, void *), void *user, void *s) override
     {
         fn(s, user);  // as the CUDA backend does: the caller enqueues nothing real here

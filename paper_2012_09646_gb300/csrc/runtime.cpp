@@ -85,6 +85,7 @@ struct StreamState {
     bool owned = true;
     int64_t tail = -1;
     int32_t active = 0;
+    int32_t kernels = 0;  // active elements other than copies
     uint64_t last_use = 0;
     bool queued = false;
 };
@@ -111,6 +112,7 @@ struct Ctx {
     std::deque<Node> nodes;
     std::vector<int64_t> parent_arena;
     int64_t active_count = 0;
+    int64_t active_kernels = 0;  // sum of the streams' kernels
     size_t trim_at = 0;  // node-table size of the next trim check
     int64_t reader_entries = 0;  // sum of the arrays' reader-set sizes
 
@@ -203,9 +205,9 @@ struct Ctx {
         return fail(r == BE_STICKY ? GDAG_ERR_POISONED : GDAG_ERR_CUDA, "%s: %s", what, be->err.c_str());
     }
 
-    void log_op(int type, int stream, int event, int64_t node)
+    void log_op(int type, int stream, int event, int64_t node, bool beside = false)
     {
-        if (opt.record_log && !capturing) op_log.push_back(gdag_op{type, stream, event, 0, node});
+        if (opt.record_log && !capturing) op_log.push_back(gdag_op{type, stream, event, beside, node});
     }
 
     // ------------------------------------------------------------- nodes
@@ -233,6 +235,14 @@ struct Ctx {
         return GDAG_OK;
     }
 
+    static bool is_copy(const Node &n)
+    {
+        return n.kind == GDAG_NODE_HOST_WRITE || n.kind == GDAG_NODE_HOST_READ || n.kind == GDAG_NODE_HOST_PREFETCH;
+    }
+    // Kernels that a copy on stream s does not follow may be running (they are
+    // not known to be complete).
+    bool kernels_beside(int32_t s) const { return active_kernels > streams[(size_t)s].kernels; }
+
     // Mark one active node inactive: its event slot and its stream's share
     // are released.  Returns false if it was not active.
     bool deactivate(Node *n)
@@ -246,6 +256,8 @@ struct Ctx {
         }
         if (n->stream >= 0) {
             StreamState &s = streams[(size_t)n->stream];
+            s.kernels -= !is_copy(*n);
+            active_kernels -= !is_copy(*n);
             if (--s.active == 0 && !s.queued) {
                 s.queued = true;
                 free_streams.push_back(n->stream);
@@ -590,6 +602,8 @@ struct Ctx {
             free_streams.erase(std::find(free_streams.begin(), free_streams.end(), s));
         }
         ss.active++;
+        ss.kernels += !is_copy(*node(id));
+        active_kernels += !is_copy(*node(id));
         ss.tail = id;
         ss.last_use = ++tick;
         if (opt.record_log == 1) node_log[node_log.size() - (size_t)(next_id() - id)].stream = s;
@@ -1233,9 +1247,10 @@ int gdag_array_write(gdag_ctx *c, gdag_array a, const void *src, size_t off, siz
     int32_t st;
     r = c->place(id, &st);
     if (r) return c->drop_failed(id, r);
-    c->log_op(GDAG_OP_COPY_H2D, st, -1, id);
+    const bool beside = c->kernels_beside(st);
+    c->log_op(GDAG_OP_COPY_H2D, st, -1, id, beside);
     ++c->st.copies;
-    r = c->be->copy_h2d(static_cast<char *>(s->dev) + off, view, bytes, c->streams[(size_t)st].handle);
+    r = c->be->copy_h2d(static_cast<char *>(s->dev) + off, view, bytes, beside, c->streams[(size_t)st].handle);
     if (r) return c->abort_node(id, r, "host-to-device copy");
     s->view_copy = id;
     s->prefetch = -1;  // the view now holds the host's data
@@ -1276,9 +1291,10 @@ int gdag_array_read(gdag_ctx *c, gdag_array a, void *dst, size_t off, size_t byt
         int32_t st;
         r = c->place(id, &st);
         if (r) return c->drop_failed(id, r);
-        c->log_op(GDAG_OP_COPY_D2H, st, -1, id);
+        const bool beside = c->kernels_beside(st);
+        c->log_op(GDAG_OP_COPY_D2H, st, -1, id, beside);
         ++c->st.copies;
-        r = c->be->copy_d2h(view, static_cast<char *>(s->dev) + off, bytes, c->streams[(size_t)st].handle);
+        r = c->be->copy_d2h(view, static_cast<char *>(s->dev) + off, bytes, beside, c->streams[(size_t)st].handle);
         if (r) return c->abort_node(id, r, "device-to-host copy");
         r = c->finish(id, st);
         if (r) return r;
@@ -1325,9 +1341,10 @@ int gdag_array_prefetch_host(gdag_ctx *c, gdag_array a, size_t off, size_t bytes
     int32_t st;
     r = c->place(id, &st);
     if (r) return c->drop_failed(id, r);
-    c->log_op(GDAG_OP_COPY_D2H, st, -1, id);
+    const bool beside = c->kernels_beside(st);
+    c->log_op(GDAG_OP_COPY_D2H, st, -1, id, beside);
     ++c->st.copies;
-    r = c->be->copy_d2h(static_cast<char *>(s->host) + off, static_cast<char *>(s->dev) + off, bytes,
+    r = c->be->copy_d2h(static_cast<char *>(s->host) + off, static_cast<char *>(s->dev) + off, bytes, beside,
                         c->streams[(size_t)st].handle);
     if (r) return c->abort_node(id, r, "device-to-host prefetch");
     s->prefetch = id;

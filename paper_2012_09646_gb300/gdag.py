@@ -98,7 +98,7 @@ class gdag_node_info(ctypes.Structure):
 
 class gdag_op(ctypes.Structure):
     _fields_ = [("type", ctypes.c_int32), ("stream", ctypes.c_int32), ("event", ctypes.c_int32),
-                ("reserved", ctypes.c_int32), ("node", ctypes.c_int64)]
+                ("beside", ctypes.c_int32), ("node", ctypes.c_int64)]
 
 
 class gdag_trace_rec(ctypes.Structure):
