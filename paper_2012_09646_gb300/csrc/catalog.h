@@ -50,11 +50,10 @@ typedef int (*LauncherFn)(const LaunchArgs &, void *stream);
 typedef int (*FusedLauncherFn)(const LaunchArgs *members, int count, void *stream);
 
 // Merged launches.  gdag_issue hands a merge rule the run of consecutive
-// built-in launches that starts at a launch of the rule's kernel (each
-// resolved and validated, with its signature's access modes and the automatic
-// launch shape).  The rule may claim several of them, run[0] among them, to be
-// issued as one unit, whose launcher does the work of all members.  The
-// runtime checks that moving the later members up to the first one's place
+// built-in launches that starts at a launch of the rule's kernel (each with its
+// signature's access modes and the automatic launch shape).  The rule may claim
+// several of them, the first one among them, to be issued as one unit, whose
+// launcher does the work of all members.  The runtime checks that moving the later members up to the first one's place
 // passes no conflicting launch, and that no array that a member writes shares
 // memory with another array of the unit.
 constexpr int kMaxRun = 32;
@@ -66,6 +65,21 @@ struct RunLaunch {
     int32_t array[kMaxArgs];  // array handles (array arguments only)
 };
 
+// A rule is asked at every launch of its kernel, so it looks at kernels and at the
+// first launch before it has others resolved: a launch's arguments are resolved
+// and validated once a gdag_issue call, when a rule first asks for them.
+class Run {
+  public:
+    // The kernel of the run's launch j; null past the run's end.
+    virtual const KernelEntry *kernel(int j) = 0;
+    // Launch j, resolved and validated with those before it; null if the run ends
+    // before.  Valid for this asking of the rule.
+    virtual const RunLaunch *at(int j) = 0;
+
+  protected:
+    ~Run() = default;
+};
+
 // As LauncherFn, over the members' arguments.
 typedef int (*MergeLaunchFn)(const LaunchArgs *const *m, int count, void *stream);
 struct Merge {
@@ -73,7 +87,7 @@ struct Merge {
     int member[kMaxRun];  // indices into the run, in the order the launcher wants them
     MergeLaunchFn launch = nullptr;
 };
-typedef bool (*MergeFn)(const RunLaunch *run, int n, Merge &out);
+typedef bool (*MergeFn)(Run &run, Merge &out);
 
 struct KernelEntry {
     std::string name;
@@ -85,6 +99,11 @@ struct KernelEntry {
     FusedLauncherFn fused = nullptr;  // built-ins with a fused form only
     MergeFn merge = nullptr;          // built-ins that start a merged launch only
 };
+
+template <size_t N> inline bool is(const KernelEntry *k, const char (&name)[N])
+{
+    return k && k->name.size() == N - 1 && std::memcmp(k->name.data(), name, N - 1) == 0;
+}
 
 // Built-in kernels (defined by the kernel translation units).
 int builtin_count();

@@ -311,16 +311,18 @@ int launch_bs_run(const LaunchArgs *const *m, int count, void *s)
 // fused form's one wave of blocks has a tail that separate launches fill).
 constexpr int64_t kBsMergeMax = 1 << 21;
 
-bool merge_bs(const RunLaunch *run, int n, Merge &out)
+bool merge_bs(Run &run, Merge &out)
 {
     out.count = 0;
-    for (int i = 0; i < n; ++i) {
-        if (run[i].k->name != "bs_call" || run[i].a.i64(2) > kBsMergeMax) break;
+    for (int i = 0; is(run.kernel(i), "bs_call"); ++i) {
+        const RunLaunch *f = run.at(i);
+        if (!f || f->a.i64(2) > kBsMergeMax) break;
         // what a member writes, no other member touches
-        bool apart = run[i].array[0] != run[i].array[1];
-        for (int j = 0; j < i; ++j)
-            apart = apart && run[i].array[1] != run[j].array[0] && run[i].array[1] != run[j].array[1] &&
-                    run[i].array[0] != run[j].array[1];
+        bool apart = f->array[0] != f->array[1];
+        for (int j = 0; j < i; ++j) {
+            const RunLaunch *g = run.at(j);
+            apart = apart && f->array[1] != g->array[0] && f->array[1] != g->array[1] && f->array[0] != g->array[1];
+        }
         if (!apart) break;
         out.member[out.count++] = i;
     }

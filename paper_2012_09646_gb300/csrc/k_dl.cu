@@ -820,16 +820,17 @@ bool apart(const RunLaunch &f, const RunLaunch &g)
 // launch of it that shares nothing written with the first.  One grid pays one
 // start-up and one part-filled last round (4096 tiles over 152 CTAs make 27
 // rounds, 2048 make 14), and the host one launch.
-template <MergeLaunchFn LAUNCH> bool merge_branches(const RunLaunch *run, int n, Merge &out)
+template <MergeLaunchFn LAUNCH> bool merge_branches(Run &run, Merge &out)
 {
-    const RunLaunch &f = run[0];
+    const RunLaunch &f = *run.at(0);
     // work items (tiles or planes), which one grid counts in 32 bits
     auto items = [](const LaunchArgs &a) {
         return a.nargs == 8 ? (int64_t)a.i32(5) * (a.i32(6) / 2) * ceil_div(a.i32(7), kTileCols) : (int64_t)a.i32(2);
     };
-    for (int j = 1; j < n; ++j) {
-        const RunLaunch &g = run[j];
-        if (g.k != f.k) continue;
+    for (int j = 1; run.kernel(j); ++j) {
+        if (run.kernel(j) != f.k) continue;
+        if (!run.at(j)) return false;
+        const RunLaunch &g = *run.at(j);
         if (items(f.a) + items(g.a) > INT32_MAX / 2 || !apart(f, g)) return false;
         out.count = 2;
         out.member[0] = 0;
@@ -860,15 +861,16 @@ int launch_branches(const LaunchArgs *const *m, int, void *s)
 
 // The five launches in a row (either order of the branches), the pools after both
 // convolutions; other programs keep the pairs.
-bool merge_dl(const RunLaunch *run, int n, Merge &out)
+bool merge_dl(Run &run, Merge &out)
 {
-    if (!merge_branches<launch_conv_run>(run, n, out)) return false;
-    if (n < 5 || out.member[1] != 1 || run[2].k->launcher != launch_avgpool || run[3].k != run[2].k ||
-        run[4].k->launcher != launch_dense)
+    if (!merge_branches<launch_conv_run>(run, out)) return false;
+    if (out.member[1] != 1 || !is(run.kernel(2), "avgpool_global") || run.kernel(3) != run.kernel(2) ||
+        !is(run.kernel(4), "concat_dense") || !run.at(4))
         return true;
-    const int pool0 = run[2].array[0] == run[0].array[3] ? 2 : 3, pool1 = 5 - pool0;
-    const RunLaunch &p = run[pool0], &q = run[pool1], &d = run[4];
-    if (p.array[0] != run[0].array[3] || q.array[0] != run[1].array[3] || !apart(p, q)) return true;
+    const RunLaunch &a = *run.at(0), &b = *run.at(1);
+    const int pool0 = run.at(2)->array[0] == a.array[3] ? 2 : 3, pool1 = 5 - pool0;
+    const RunLaunch &p = *run.at(pool0), &q = *run.at(pool1), &d = *run.at(4);
+    if (p.array[0] != a.array[3] || q.array[0] != b.array[3] || !apart(p, q)) return true;
     if (!((d.array[0] == p.array[1] && d.array[1] == q.array[1]) || (d.array[0] == q.array[1] && d.array[1] == p.array[1])))
         return true;
     if ((int64_t)p.a.i32(2) + q.a.i32(2) > INT32_MAX / 2) return true;

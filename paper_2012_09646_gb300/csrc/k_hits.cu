@@ -716,19 +716,20 @@ int launch_seg_scale(const LaunchArgs &a, void *s)
 // graphs the two branches on two streams are the quicker form where one program
 // has the device (1e6 rows 287 us against 314, 1e7 2160 against 2234): a branch's
 // norm and scaling run beside the other's product.
-template <MergeLaunchFn LAUNCH> bool merge_two(const RunLaunch *run, int n, Merge &out)
+template <MergeLaunchFn LAUNCH> bool merge_two(Run &run, Merge &out)
 {
-    const RunLaunch &f = run[0];
+    const RunLaunch &f = *run.at(0);
     auto small = [](const RunLaunch &l) {
-        const std::string &k = l.k->name;
-        if (k == "spmv_csr") return (int64_t)l.a.i32(7) + l.a.i32(8) <= (1 << 22);
-        return (k == "l2norm" ? l.a.i64(3) : k == "scale" ? l.a.i64(2) : (int64_t)l.a.i32(k == "seg_l2norm" ? 5 : 4)) <=
-               (1 << 20);
+        if (is(l.k, "spmv_csr")) return (int64_t)l.a.i32(7) + l.a.i32(8) <= (1 << 22);
+        return (is(l.k, "l2norm")  ? l.a.i64(3)
+                : is(l.k, "scale") ? l.a.i64(2)
+                                   : (int64_t)l.a.i32(is(l.k, "seg_l2norm") ? 5 : 4)) <= (1 << 20);
     };
     if (!small(f)) return false;
-    for (int j = 1; j < n; ++j) {
-        const RunLaunch &g = run[j];
-        if (g.k != f.k) continue;
+    for (int j = 1; run.kernel(j); ++j) {
+        if (run.kernel(j) != f.k) continue;
+        if (!run.at(j)) return false;
+        const RunLaunch &g = *run.at(j);
         if (!small(g)) return false;
         // what either writes, the other does not touch
         bool apart = true;

@@ -542,7 +542,7 @@ KernelEntry entry(const char *name, const void *fn, std::initializer_list<gdag_a
 
 }  // namespace
 
-bool merge_img(const RunLaunch *run, int n, Merge &out);  // k_img_merge.cu
+bool merge_img(Run &run, Merge &out);  // k_img_merge.cu
 
 void append_img_kernels(std::vector<KernelEntry> &v)
 {

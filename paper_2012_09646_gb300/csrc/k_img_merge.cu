@@ -586,12 +586,14 @@ int launch_img_merged(const LaunchArgs *const *m, int, void *sv)
     return vec ? launch_stages<true>(m, (cudaStream_t)sv) : launch_stages<false>(m, (cudaStream_t)sv);
 }
 
-// the first launch of `kernel` in the run whose array arguments named by
+// the first launch of `kernel` among the run's first n whose array arguments named by
 // (index, handle) pairs match; -1 if there is none
-int find(const RunLaunch *run, int n, const char *kernel, int i0, int h0, int i1, int h1)
+template <size_t N> int find(Run &run, int n, const char (&kernel)[N], int i0, int h0, int i1, int h1)
 {
-    for (int j = 0; j < n; ++j)
-        if (run[j].array[i0] == h0 && (i1 < 0 || run[j].array[i1] == h1) && run[j].k->name == kernel) return j;
+    for (int j = 0; j < n; ++j) {
+        const RunLaunch &l = *run.at(j);
+        if (l.array[i0] == h0 && (i1 < 0 || l.array[i1] == h1) && is(l.k, kernel)) return j;
+    }
     return -1;
 }
 
@@ -599,19 +601,20 @@ int find(const RunLaunch *run, int n, const char *kernel, int i0, int h0, int i1
 
 // The IMG program around the combine launch of the run: found by its data
 // flow, whatever the order of its independent launches.
-bool merge_img(const RunLaunch *run, int n, Merge &out)
+bool merge_img(Run &run, Merge &out)
 {
-    int c = -1;
-    for (int j = 0; j < n && c < 0; ++j)
-        if (run[j].k->name == "combine") c = j;
-    if (c < 0) return false;
-    const int32_t s = run[c].array[0], ba = run[c].array[1], bb = run[c].array[2], ea = run[c].array[3],
-                  eb = run[c].array[4];
+    int c = 1;
+    while (run.kernel(c) && !is(run.kernel(c), "combine")) ++c;
+    if (c + 1 < kRoles || !run.kernel(c) || !run.at(c)) return false;
+    const int n = c + 1;
+    auto at = [&](int j) -> const RunLaunch & { return *run.at(j); };
+    const int32_t s = at(c).array[0], ba = at(c).array[1], bb = at(c).array[2], ea = at(c).array[3],
+                  eb = at(c).array[4];
     int *r = out.member;
     r[kCombine] = c;
     r[kUnsharp] = find(run, n, "unsharp", 1, ba, 2, s);
     if (r[kUnsharp] < 0) return false;
-    const int32_t img = run[r[kUnsharp]].array[0];
+    const int32_t img = at(r[kUnsharp]).array[0];
     r[kBlurA] = find(run, n, "gauss_blur", 0, img, 1, ba);
     r[kBlurB] = find(run, n, "gauss_blur", 0, img, 1, bb);
     r[kSobelA] = find(run, n, "sobel", 0, ba, 1, ea);
@@ -620,8 +623,8 @@ bool merge_img(const RunLaunch *run, int n, Merge &out)
     r[kMmB] = find(run, n, "minmax", 0, eb, -1, 0);
     for (int q = 0; q < kRoles; ++q)
         if (q != kExtA && q != kExtB && r[q] < 0) return false;
-    r[kExtA] = find(run, n, "extend", 0, ea, 1, run[r[kMmA]].array[1]);
-    r[kExtB] = find(run, n, "extend", 0, eb, 1, run[r[kMmB]].array[1]);
+    r[kExtA] = find(run, n, "extend", 0, ea, 1, at(r[kMmA]).array[1]);
+    r[kExtB] = find(run, n, "extend", 0, eb, 1, at(r[kMmB]).array[1]);
     if (r[kExtA] < 0 || r[kExtB] < 0) return false;
     // each launch after those whose results it takes, before those that
     // overwrite what it reads
@@ -631,24 +634,24 @@ bool merge_img(const RunLaunch *run, int n, Merge &out)
     for (const auto &p : before)
         if (r[p[0]] >= r[p[1]]) return false;
     // what is written is written once, and is none of the inputs
-    const int32_t w[] = {ba, bb, ea, eb, s, run[c].array[5], run[r[kMmA]].array[1], run[r[kMmB]].array[1],
-                         run[r[kMmA]].array[2], run[r[kMmB]].array[2], img, run[r[kBlurA]].array[2],
-                         run[r[kBlurB]].array[2]};
+    const int32_t w[] = {ba, bb, ea, eb, s, at(c).array[5], at(r[kMmA]).array[1], at(r[kMmB]).array[1],
+                         at(r[kMmA]).array[2], at(r[kMmB]).array[2], img, at(r[kBlurA]).array[2],
+                         at(r[kBlurB]).array[2]};
     for (int i = 0; i < 10; ++i)
         for (int j = i + 1; j < 13; ++j)
             if (w[i] == w[j]) return false;
     // one image size, and radii that stage 1 is built for
-    const LaunchArgs &l = run[r[kBlurA]].a;
+    const LaunchArgs &l = at(r[kBlurA]).a;
     const int rows = l.i32(3), cols = l.i32(4);
     const int64_t px = (int64_t)rows * cols;
     for (int q : {kBlurB})
-        if (run[r[q]].a.i32(3) != rows || run[r[q]].a.i32(4) != cols) return false;
+        if (at(r[q]).a.i32(3) != rows || at(r[q]).a.i32(4) != cols) return false;
     for (int q : {kSobelA, kSobelB})
-        if (run[r[q]].a.i32(2) != rows || run[r[q]].a.i32(3) != cols) return false;
-    if (run[r[kMmA]].a.i64(3) != px || run[r[kMmB]].a.i64(3) != px || run[r[kExtA]].a.i64(2) != px ||
-        run[r[kExtB]].a.i64(2) != px || run[r[kUnsharp]].a.i64(4) != px || run[c].a.i64(6) != px)
+        if (at(r[q]).a.i32(2) != rows || at(r[q]).a.i32(3) != cols) return false;
+    if (at(r[kMmA]).a.i64(3) != px || at(r[kMmB]).a.i64(3) != px || at(r[kExtA]).a.i64(2) != px ||
+        at(r[kExtB]).a.i64(2) != px || at(r[kUnsharp]).a.i64(4) != px || at(c).a.i64(6) != px)
         return false;
-    const int ra = l.i32(5), rb = run[r[kBlurB]].a.i32(5);
+    const int ra = l.i32(5), rb = at(r[kBlurB]).a.i32(5);
     if (ra >= rb || rb > kMergeMaxR) return false;
     // the pairs of the tallest bands fit the minmax scratch
     if (ceil_div(cols, kMgCols) * ceil_div(ceil_div(rows, kS1MaxBand), kStWarps) > kMmMaxBlocks) return false;

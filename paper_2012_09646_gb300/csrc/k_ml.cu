@@ -423,7 +423,7 @@ __global__ void __launch_bounds__(256) argmax_combine_kernel(const float *__rest
 // the tcgen05 form (k_ml_tc.cu): classes <= 16, feats a multiple of 64 up to 1024
 bool scores_tc_ok(int feats, int classes);
 int launch_scores_tc(const LaunchArgs &a, cudaStream_t s);
-bool merge_scores(const RunLaunch *run, int n, Merge &out);
+bool merge_scores(Run &run, Merge &out);
 
 namespace {
 
@@ -613,20 +613,22 @@ int launch_softmax_argmax(const LaunchArgs *const *m, int, void *s)
 // against 71.8).
 constexpr int kTailRows = 32768;
 
-bool merge_softmax(const RunLaunch *run, int n, Merge &out)
+bool merge_softmax(Run &run, Merge &out)
 {
+    if (run.at(0)->a.i32(1) > kTailRows) return false;
     int r = 1;
-    while (r < n && run[r].k->name != "argmax_combine") ++r;
-    if (r == n) return false;
-    const int32_t s1 = run[r].array[0], s2 = run[r].array[1], lab = run[r].array[2], first = run[0].array[0];
-    const int rows = run[r].a.i32(3), classes = run[r].a.i32(4);
+    while (run.kernel(r) && !is(run.kernel(r), "argmax_combine")) ++r;
+    const RunLaunch *arg = run.kernel(r) ? run.at(r) : nullptr;
+    if (!arg) return false;
+    const int32_t s1 = arg->array[0], s2 = arg->array[1], lab = arg->array[2], first = run.at(0)->array[0];
+    const int rows = arg->a.i32(3), classes = arg->a.i32(4);
     if (s1 == s2 || lab == s1 || lab == s2 || (first != s1 && first != s2) || rows > kTailRows) return false;
     const int32_t other = first == s1 ? s2 : s1;
     int q = 1;
-    while (q < r && !(run[q].k->name == "row_softmax" && run[q].array[0] == other)) ++q;
+    while (q < r && !(is(run.kernel(q), "row_softmax") && run.at(q)->array[0] == other)) ++q;
     if (q == r) return false;
     for (int i : {0, q})
-        if (run[i].a.i32(1) != rows || run[i].a.i32(2) != classes) return false;
+        if (run.at(i)->a.i32(1) != rows || run.at(i)->a.i32(2) != classes) return false;
     out.count = 3;
     out.member[0] = 0;
     out.member[1] = q;

@@ -617,13 +617,15 @@ MergeLaunchFn scores_cuda_pair(int rows, int feats, int classes0, int classes1);
 
 // Two dense_scores launches over the same X (the two classifiers of the ML
 // program).
-bool merge_scores(const RunLaunch *run, int n, Merge &out)
+bool merge_scores(Run &run, Merge &out)
 {
-    const RunLaunch &f = run[0];
+    const RunLaunch &f = *run.at(0);
     const int rows = f.a.i32(4), feats = f.a.i32(5), c0 = f.a.i32(6);
-    for (int j = 1; j < n; ++j) {
-        const RunLaunch &g = run[j];
-        if (g.k->name != "dense_scores" || g.array[0] != f.array[0]) continue;
+    for (int j = 1; run.kernel(j); ++j) {
+        if (run.kernel(j) != f.k) continue;
+        if (!run.at(j)) return false;
+        const RunLaunch &g = *run.at(j);
+        if (g.array[0] != f.array[0]) continue;
         if (g.a.i32(4) != rows || g.a.i32(5) != feats) continue;
         const int c1 = g.a.i32(6);
         const bool t0 = scores_tc_ok(feats, c0), t1 = scores_tc_ok(feats, c1);

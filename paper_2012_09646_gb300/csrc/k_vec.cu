@@ -356,18 +356,19 @@ int launch_square_reduce(const LaunchArgs *const *m, int, void *s)
 // The run's first launch squares an array that the first vec_reduce_diff after
 // it takes, with the other array's square between.  Every element of both is
 // squared and summed, and the four arrays are different ones.
-bool merge_vec(const RunLaunch *run, int n, Merge &out)
+bool merge_vec(Run &run, Merge &out)
 {
     int r = 1;
-    while (r < n && run[r].k->name != "vec_reduce_diff") ++r;
-    if (r == n) return false;
-    const int32_t x = run[r].array[0], y = run[r].array[1], z = run[r].array[2], sc = run[r].array[3];
-    const int32_t first = run[0].array[0], other = first == x ? y : x;
+    while (run.kernel(r) && !is(run.kernel(r), "vec_reduce_diff")) ++r;
+    const RunLaunch *red = run.kernel(r) ? run.at(r) : nullptr;
+    if (!red) return false;
+    const int32_t x = red->array[0], y = red->array[1], z = red->array[2], sc = red->array[3];
+    const int32_t first = run.at(0)->array[0], other = first == x ? y : x;
     if ((first != x && first != y) || x == y || z == x || z == y || sc == x || sc == y || sc == z) return false;
     int q = 1;
-    while (q < r && !(run[q].k->name == "vec_square" && run[q].array[0] == other)) ++q;
-    const int64_t len = run[r].a.i64(4);
-    if (q == r || run[0].a.i64(1) != len || run[q].a.i64(1) != len) return false;
+    while (q < r && !(is(run.kernel(q), "vec_square") && run.at(q)->array[0] == other)) ++q;
+    const int64_t len = red->a.i64(4);
+    if (q == r || run.at(0)->a.i64(1) != len || run.at(q)->a.i64(1) != len) return false;
     out.count = 3;
     out.member[0] = 0;
     out.member[1] = q;

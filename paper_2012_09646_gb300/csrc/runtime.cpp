@@ -95,6 +95,16 @@ struct Access {
     int32_t bits;
 };
 
+// A launch element of a gdag_issue call as the merge rules see it.
+struct Resolved {
+    int32_t elem = -1;
+    bool ok;
+    gdag::RunLaunch l;
+    Access acc[gdag::kMaxArgs];
+    int nacc;
+};
+constexpr int kResolvedRing = 64;
+
 }  // namespace
 
 struct Ctx {
@@ -135,6 +145,7 @@ struct Ctx {
     // scratch for one element or one call
     std::vector<int64_t> par, retire_stack, ext;
     std::vector<uint8_t> issued_early;
+    std::vector<Resolved> resolved;  // kResolvedRing once used
 
     // stream capture (CUDA graphs of a repeated DAG shape)
     bool capturing = false;
@@ -772,6 +783,8 @@ struct IssueRange {
 };
 
 using gdag::Access;
+using gdag::Resolved;
+using gdag::kResolvedRing;
 using gdag::ArrayState;
 using gdag::Ctx;
 using gdag::KernelEntry;
@@ -1047,6 +1060,9 @@ static int resolve(gdag_ctx *c, gdag_kernel k, gdag_dim3 grid, gdag_dim3 block, 
     return GDAG_OK;
 }
 
+static int issue_launch(gdag_ctx *c, gdag_kernel k, const LaunchArgs &la, const Access *acc, int nacc,
+                        int64_t *node_out);
+
 int gdag_launch(gdag_ctx *c, gdag_kernel k, gdag_dim3 grid, gdag_dim3 block, size_t smem, const gdag_arg *args,
                 int32_t nargs, int64_t *node_out)
 {
@@ -1059,6 +1075,22 @@ int gdag_launch(gdag_ctx *c, gdag_kernel k, gdag_dim3 grid, gdag_dim3 block, siz
     int nacc;
     r = resolve(c, k, grid, block, smem, args, nargs, la, acc, &nacc);
     if (r) return r;
+    return issue_launch(c, k, la, acc, nacc, node_out);
+}
+
+// gdag_launch of a launch that is resolved already.
+static int launch_resolved(gdag_ctx *c, gdag_kernel k, const LaunchArgs &la, const Access *acc, int nacc,
+                           int64_t *node_out)
+{
+    int r = c->guard();
+    if (r) return r;
+    IssueRange nvtx(c, c->kernels[(size_t)k].name.c_str());
+    return issue_launch(c, k, la, acc, nacc, node_out);
+}
+
+static int issue_launch(gdag_ctx *c, gdag_kernel k, const LaunchArgs &la, const Access *acc, int nacc, int64_t *node_out)
+{
+    int r;
     c->capture_note(acc, nacc);
     int64_t id = c->next_id();
     c->infer(id, acc, nacc);
@@ -1363,29 +1395,33 @@ static bool elem_args_ok(const gdag_elem &e, int64_t nargs_total)
            (int64_t)e.nargs * count <= nargs_total - e.arg0;
 }
 
-// Resolve launch element e for a merge rule: a built-in kernel with the
-// automatic shape and its signature's access modes, valid as it stands.
-// False (with the context's last error restored) ends the run.
-static bool run_launch(gdag_ctx *c, const gdag_elem &e, const gdag_arg *args, int64_t nargs_total,
-                       gdag::RunLaunch &out, Access *acc, int *nacc)
+// Launch element i for a merge rule: a built-in kernel with the automatic shape
+// and its signature's access modes, valid as it stands (with the context's last
+// error restored).  Resolved once a call: the ring holds the elements that the
+// runs since then looked at.
+static const Resolved &resolved(gdag_ctx *c, const gdag_elem *elems, int32_t i, const gdag_arg *args,
+                                int64_t nargs_total)
 {
-    if (e.type != GDAG_ELEM_LAUNCH || e.smem || e.grid.x || e.grid.y || e.grid.z || !elem_args_ok(e, nargs_total))
-        return false;
-    if (e.kernel < 0 || (size_t)e.kernel >= c->kernels.size() || !c->kernels[(size_t)e.kernel].launcher) return false;
+    Resolved &out = c->resolved[(size_t)i % kResolvedRing];
+    if (out.elem == i) return out;
+    out.elem = i;
+    out.ok = false;
+    const gdag_elem &e = elems[i];
+    if (e.smem || e.grid.x || e.grid.y || e.grid.z || !elem_args_ok(e, nargs_total)) return out;
     const KernelEntry &k = c->kernels[(size_t)e.kernel];
     const gdag_arg *a = e.nargs ? args + e.arg0 : nullptr;
-    if (e.nargs != k.nargs) return false;
-    std::fill(out.array, out.array + gdag::kMaxArgs, -1);
-    for (int i = 0; i < e.nargs; ++i) {
-        if (a[i].kind == GDAG_ARG_ARRAY && a[i].mode != GDAG_MODE_SIGNATURE && a[i].mode != k.spec[i].mode) return false;
-        if (a[i].kind == GDAG_ARG_ARRAY) out.array[i] = a[i].array;
+    if (e.nargs != k.nargs) return out;
+    std::fill(out.l.array, out.l.array + gdag::kMaxArgs, -1);
+    for (int j = 0; j < e.nargs; ++j) {
+        if (a[j].kind == GDAG_ARG_ARRAY && a[j].mode != GDAG_MODE_SIGNATURE && a[j].mode != k.spec[j].mode) return out;
+        if (a[j].kind == GDAG_ARG_ARRAY) out.l.array[j] = a[j].array;
     }
     std::string kept;
     kept.swap(c->last_error);
-    const bool ok = resolve(c, e.kernel, e.grid, e.block, 0, a, e.nargs, out.a, acc, nacc) == GDAG_OK;
+    out.ok = resolve(c, e.kernel, e.grid, e.block, 0, a, e.nargs, out.l.a, out.acc, &out.nacc) == GDAG_OK;
     kept.swap(c->last_error);
-    out.k = &k;
-    return ok;
+    out.l.k = &k;
+    return out;
 }
 
 static bool conflicting(const Access *a, int na, const Access *b, int nb)
@@ -1396,17 +1432,58 @@ static bool conflicting(const Access *a, int na, const Access *b, int nb)
     return false;
 }
 
-// The run of launches that starts at element i (elements already issued as
+// The run of launches that starts at element `first` (elements already issued as
 // members of an earlier unit are passed over), and what its first launch's
-// rule makes of it.
-struct MergeRun {
-    gdag::RunLaunch run[gdag::kMaxRun];
-    Access acc[gdag::kMaxRun][gdag::kMaxArgs];
-    int nacc[gdag::kMaxRun];
-    int32_t elem[gdag::kMaxRun];
+// rule makes of it.  It ends before the element whose place in the ring the first
+// one has.
+struct MergeRun final : gdag::Run {
+    gdag_ctx *c;
+    const gdag_elem *elems;
+    const gdag_arg *args;
+    int64_t nargs_total;
+    int32_t end;
+    int32_t elem[gdag::kMaxRun];              // the run's launches so far
+    int known = 1;
+    bool ended = false;
+    const Resolved *r[gdag::kMaxRun];         // those resolved so far
     int n = 0;
     gdag::Merge m;
     int order[gdag::kMaxRun];  // the members in the run's order
+
+    MergeRun(gdag_ctx *ctx, const gdag_elem *e, int32_t ne, const gdag_arg *a, int64_t na, int32_t first)
+        : c(ctx), elems(e), args(a), nargs_total(na), end(std::min<int64_t>(ne, (int64_t)first + kResolvedRing))
+    {
+        elem[0] = first;
+    }
+    const KernelEntry *kernel(int j) override
+    {
+        while (known <= j && !ended) {
+            int32_t i = elem[known - 1] + 1;
+            while (i < end && !c->issued_early.empty() && c->issued_early[(size_t)i]) ++i;
+            if (known == gdag::kMaxRun || i >= end || elems[i].type != GDAG_ELEM_LAUNCH || elems[i].kernel < 0 ||
+                (size_t)elems[i].kernel >= c->kernels.size() || !c->kernels[(size_t)elems[i].kernel].launcher)
+                ended = true;
+            else
+                elem[known++] = i;
+        }
+        return j < known ? &c->kernels[(size_t)elems[elem[j]].kernel] : nullptr;
+    }
+    const gdag::RunLaunch *at(int j) override
+    {
+        while (n <= j) {
+            if (!kernel(n)) return nullptr;
+            const Resolved &x = resolved(c, elems, elem[n], args, nargs_total);
+            if (!x.ok) {
+                known = n;
+                ended = true;
+                return nullptr;
+            }
+            r[n++] = &x;
+        }
+        return &r[j]->l;
+    }
+    const Access *acc(int j) const { return r[j]->acc; }
+    int nacc(int j) const { return r[j]->nacc; }
 };
 
 // The checks a rule leaves to the runtime.
@@ -1425,7 +1502,7 @@ static bool merge_legal(gdag_ctx *c, MergeRun &q)
     // a member moves up past every launch between it and the first one
     for (int k = 1; k < m.count; ++k)
         for (int j = 0, x = q.order[k]; j < x; ++j)
-            if (!in[j] && conflicting(q.acc[j], q.nacc[j], q.acc[x], q.nacc[x])) return false;
+            if (!in[j] && conflicting(q.acc(j), q.nacc(j), q.acc(x), q.nacc(x))) return false;
     // what a member writes shares no memory with any other array of the unit
     // (other handles may name the same memory: the members would no longer
     // run one after another on it)
@@ -1436,8 +1513,8 @@ static bool merge_legal(gdag_ctx *c, MergeRun &q)
     } span[gdag::kMaxRun * gdag::kMaxArgs];
     int ns = 0;
     for (int k = 0; k < m.count; ++k)
-        for (int x = 0, mem = q.order[k]; x < q.nacc[mem]; ++x) {
-            const Access &w = q.acc[mem][x];
+        for (int x = 0, mem = q.order[k]; x < q.nacc(mem); ++x) {
+            const Access &w = q.acc(mem)[x];
             int i = 0;
             while (i < ns && span[i].array != w.array) ++i;
             if (i == ns) {
@@ -1466,14 +1543,14 @@ static int issue_merged(gdag_ctx *c, const MergeRun &q, const gdag_elem *elems, 
     ext.clear();
     for (int k = 0; k < m.count; ++k) {
         const int x = q.order[k];
-        la[k] = &q.run[m.member[k]].a;
-        c->capture_note(q.acc[x], q.nacc[x]);
+        la[k] = &q.r[m.member[k]]->l.a;
+        c->capture_note(q.acc(x), q.nacc(x));
         const int64_t id = c->next_id();
-        c->infer(id, q.acc[x], q.nacc[x]);
+        c->infer(id, q.acc(x), q.nacc(x));
         for (int64_t p : c->par)
             if (p < first) ext.push_back(p);
-        for (int i = 0; i < q.nacc[x]; ++i)
-            if (q.acc[x][i].bits & gdag::W_BIT) c->arrays[(size_t)q.acc[x][i].array].host_valid = false;
+        for (int i = 0; i < q.nacc(x); ++i)
+            if (q.acc(x)[i].bits & gdag::W_BIT) c->arrays[(size_t)q.acc(x)[i].array].host_valid = false;
         c->push_node(GDAG_NODE_KERNEL);
         c->node(id)->label = elems[q.elem[x]].kernel;
         c->activate(id);
@@ -1509,7 +1586,7 @@ static int issue_merged(gdag_ctx *c, const MergeRun &q, const gdag_elem *elems, 
     const int64_t last = ids[m.count - 1];
     c->log_op(GDAG_OP_LAUNCH, s, -1, last);
     ++c->st.launches;
-    r = c->be->launch_merged(m, la, q.run[0].k->name.c_str(), c->streams[(size_t)s].handle);
+    r = c->be->launch_merged(m, la, q.r[0]->l.k->name.c_str(), c->streams[(size_t)s].handle);
     if (r) return drop(c->be_fail(r, "merged launch"), s);  // some of its kernels may be running
     r = c->record_end(last, s);
     if (r) return drop(r, s);
@@ -1532,6 +1609,10 @@ static int issue_each(gdag_ctx *c, const gdag_elem *elems, int32_t n, const gdag
     const bool merging = c->opt.policy == GDAG_POLICY_PARALLEL && !c->opt.trace && !c->poisoned;
     std::vector<uint8_t> &done = c->issued_early;  // elements issued as members of an earlier unit
     done.clear();
+    if (merging) {
+        c->resolved.resize(kResolvedRing);
+        for (Resolved &x : c->resolved) x.elem = -1;
+    }
     for (int32_t i = 0; i < n; ++i) {
         const gdag_elem &e = elems[i];
         if (!done.empty() && done[(size_t)i]) {
@@ -1540,13 +1621,8 @@ static int issue_each(gdag_ctx *c, const gdag_elem *elems, int32_t n, const gdag
         }
         if (merging && e.type == GDAG_ELEM_LAUNCH && i + 1 < n && e.kernel >= 0 &&
             (size_t)e.kernel < c->kernels.size() && c->kernels[(size_t)e.kernel].merge) {
-            MergeRun q;
-            for (int32_t j = i; j < n && q.n < gdag::kMaxRun; ++j) {
-                if (!done.empty() && done[(size_t)j]) continue;
-                if (!run_launch(c, elems[j], args, nargs_total, q.run[q.n], q.acc[q.n], &q.nacc[q.n])) break;
-                q.elem[q.n++] = j;
-            }
-            if (q.n > 1 && q.run[0].k->merge(q.run, q.n, q.m) && merge_legal(c, q)) {
+            MergeRun q(c, elems, n, args, nargs_total, i);
+            if (q.at(0) && q.r[0]->l.k->merge(q, q.m) && merge_legal(c, q)) {
                 int64_t ids[gdag::kMaxRun];
                 const int r = issue_merged(c, q, elems, ids);
                 if (done.empty()) done.resize((size_t)n, 0);
@@ -1572,7 +1648,10 @@ static int issue_each(gdag_ctx *c, const gdag_elem *elems, int32_t n, const gdag
                 break;
             }
             const gdag_arg *a = e.nargs ? args + e.arg0 : nullptr;
-            if (e.type == GDAG_ELEM_LAUNCH)
+            const Resolved *x = merging ? &c->resolved[(size_t)i % kResolvedRing] : nullptr;
+            if (x && x->elem == i && x->ok)  // a rule has looked at it
+                r = launch_resolved(c, e.kernel, x->l.a, x->acc, x->nacc, &node);
+            else if (e.type == GDAG_ELEM_LAUNCH)
                 r = gdag_launch(c, e.kernel, e.grid, e.block, (size_t)e.smem, a, e.nargs, &node);
             else
                 r = gdag_launch_fused(c, e.kernel, a, e.nargs, e.count, &node);

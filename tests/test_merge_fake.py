@@ -3,6 +3,7 @@ programs merge, and that merging leaves the DAG as it is: the same elements
 and edges as the single calls, every conflicting pair ordered."""
 import itertools
 import random
+import time
 
 import pytest
 
@@ -387,3 +388,58 @@ def test_a_launch_that_fails_is_waited_for_on_its_stream(merged):
     assert ops == [(G.GDAG_OP_LAUNCH, 0), (G.GDAG_OP_STREAM_SYNC, 0)]
     assert ctx.stats()["active"] == 0
     ctx.close()
+
+
+@pytest.mark.parametrize("name", ["books", "scale", "gauss_blur", "vec_square", "row_softmax"])
+def test_launches_that_do_not_merge_cost_about_as_much_to_issue(name):
+    """A list of launches whose kernel has a rule that claims none of them: each is
+    resolved once, not once for every launch before it.  Against the serial policy,
+    which asks no rule (host time, the best of many issues)."""
+    n, at = 3_000_000, itertools.count(1)
+
+    def best(policy):
+        ctx = G.Context(backend="fake", policy=policy, fake_complete=True, retire_by_query=True, trim_nodes=64)
+        arr = lambda nb: ctx.array(dev=next(at) << 30, nbytes=nb)  # noqa: E731
+        p = ctx.program()
+        for _ in range(32):
+            p.launch(*{"books": lambda: ("bs_call", arr(4 * n), arr(4 * n), n, 60.0, 0.1, 0.2, 1.0),
+                       "scale": lambda: ("scale", arr(4 * n), arr(4), n),
+                       "gauss_blur": lambda: ("gauss_blur", arr(4 * PX), arr(4 * PX), arr(20), ROWS, COLS, 2),
+                       "vec_square": lambda: ("vec_square", arr(4000), 1000),
+                       "row_softmax": lambda: ("row_softmax", arr(40000), 1000, 10)}[name]())
+        t = []
+        for _ in range(40):
+            t0 = time.perf_counter()
+            for _ in range(20):
+                p.issue()
+            t.append(time.perf_counter() - t0)
+        assert ctx.stats()["launches"] == 40 * 20 * 32
+        ctx.close()
+        return min(t)
+    # 3 to 4 times with the run resolved anew at every launch, 1.05 to 1.6 so
+    assert best(G.GDAG_POLICY_PARALLEL) <= 2.2 * best(G.GDAG_POLICY_SERIAL_ASYNC)
+
+
+def test_a_run_longer_than_the_rules_look_ahead():
+    """More launches than the ring of resolved ones holds, some of them issued early."""
+    ctx = G.Context(backend="fake", record_log=True)
+    one = G.Context(backend="fake", record_log=True)
+
+    def seq(c):
+        at = itertools.count(1)
+        arr = lambda nb: c.array(dev=next(at) << 24, nbytes=nb)  # noqa: E731
+        out = []
+        for i in range(150):
+            x, y, w = arr(400), arr(400), arr(400)
+            out += [("vec_square", x, 100), ("scale", w, arr(4), 100), ("vec_square", y, 100)]
+            if i % 3:
+                out.append(("vec_reduce_diff", x, y, arr(4), arr(G.gdag_scratch_bytes("vec_reduce_diff", 100)), 100))
+        return out
+    L = seq(ctx)
+    nodes, n = issue(ctx, L)
+    single_nodes = [one.launch(k, *a) for k, *a in seq(one)]
+    assert edges_by_position(ctx, nodes) == edges_by_position(one, single_nodes)
+    assert sorted(nodes) == list(range(len(L)))
+    assert n == 100 + 100 + 75  # sums with their squares, squares alone, pairs of scalings
+    ctx.close()
+    one.close()
