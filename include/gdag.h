@@ -483,8 +483,10 @@ int gdag_launch_external(gdag_ctx *ctx, void (*fn)(void *stream, void *user),
  * the nodes inside the call, may differ from the single calls'.  A launch
  * joins a unit only if every launch it would overtake touches nothing that it
  * writes and writes nothing that it touches.  If a unit fails, all its
- * members fail: *issued counts the elements before its first one, and
- * nodes_out names the later elements that an earlier unit had issued already.
+ * members fail: *issued counts the elements before its first one.  After a
+ * failure at element f = *issued, an element j > f was issued (by an earlier
+ * unit) if and only if nodes_out[j] >= 0 and nodes_out[f] is -1 or greater than
+ * nodes_out[j]; the other members of a unit that failed have greater nodes.
  * The units:
  *   vec_square x 2, vec_reduce_diff of the same two arrays;
  *   independent bs_call launches of up to 2^21 options each;
@@ -526,7 +528,8 @@ typedef struct {
  * number of elements handled before the first failure (n on success).  On
  * a failure the call returns that element's error at once: the elements
  * before it stay issued, the failing one behaves as its single call does
- * on that error, and the ones after it are not issued.  Never blocks the
+ * on that error, and the ones after it are not issued, except those that an
+ * earlier merged launch (above) had taken.  Never blocks the
  * host except where a single call would (policy SERIAL_SYNC, prefetch = 0,
  * both staging uses of a view in flight).  Errors: INVALID (an element
  * type, index range, or anything its single call rejects), CUDA, TIMEOUT,

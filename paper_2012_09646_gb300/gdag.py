@@ -366,6 +366,13 @@ def gdag_nodes_query(ctx, nodes):
     return done
 
 
+def _remaining(issued, nodes):
+    """The elements that a failed gdag_issue did not issue: from the failing one
+    on, those without a node or with one no older than the failing element's."""
+    fail = nodes[issued] if issued < len(nodes) else -1
+    return [j for j in range(issued, len(nodes)) if nodes[j] < 0 or 0 <= fail <= nodes[j]]
+
+
 def gdag_issue(ctx, elems, args):
     """Issue a ctypes array of gdag_elem against a ctypes array of gdag_arg;
     returns the node ids (-1 where an element made none)."""
@@ -379,6 +386,7 @@ def gdag_issue(ctx, elems, args):
         e = GdagError(r, (lib().gdag_last_error(ctx) or b"").decode(errors="replace"))
         e.issued = issued.value
         e.nodes = [nodes[i] for i in range(n)]
+        e.remaining = _remaining(e.issued, e.nodes)
         raise e
     return [nodes[i] for i in range(n)]
 
@@ -895,8 +903,10 @@ class Program:
     def issue(self, **values):
         """Bind every Param and issue all elements in one call; returns the
         node id of each element (-1 where it made none).  A failure raises
-        GdagError with ``issued`` (elements issued before the failing one)
-        and ``nodes``."""
+        GdagError with ``issued`` (elements issued before the failing one),
+        ``nodes``, and ``remaining``: the elements that were not issued, in
+        order, the failed one first.  (A later element may have been issued
+        already, in a unit with an earlier one.)"""
         if self._ready is None:
             self._prepare()
         call, plan, nodes, issued, n, _, _ = self._ready
@@ -913,6 +923,7 @@ class Program:
         if r < 0:
             e = GdagError(r, self.ctx.last_error)
             e.issued, e.nodes = issued.value, out
+            e.remaining = _remaining(e.issued, out)
             raise e
         return out
 

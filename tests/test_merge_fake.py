@@ -443,3 +443,35 @@ def test_a_run_longer_than_the_rules_look_ahead():
     assert n == 100 + 100 + 75  # sums with their squares, squares alone, pairs of scalings
     ctx.close()
     one.close()
+
+
+@pytest.mark.parametrize("fail", range(0, 12))
+def test_what_remains_after_a_failure_can_be_issued(fail):
+    """Units that take later elements with them, an element between, and a failure
+    at each operation: issuing what `remaining` names completes the program."""
+    def make(ctx):
+        at = itertools.count(1)
+        a = [ctx.array(dev=next(at) << 24, nbytes=400) for _ in range(8)]
+        z = [ctx.array(dev=next(at) << 24, nbytes=4) for _ in range(2)]
+        s = [ctx.array(dev=next(at) << 24, nbytes=G.gdag_scratch_bytes("vec_reduce_diff", 100)) for _ in range(2)]
+        return [("vec_square", a[0], 100), ("scale", a[4], z[1], 100), ("unsharp", a[5], a[6], a[7], 0.5, 100),
+                ("vec_square", a[1], 100), ("scale", a[6], z[1], 100),
+                ("vec_reduce_diff", a[0], a[1], z[0], s[0], 100), ("vec_square", a[2], 100)]
+    whole = G.Context(backend="fake")
+    _, launches = issue(whole, make(whole))
+    whole.close()
+    ctx = G.Context(backend="fake", fake_fail_op=fail, record_log=True)
+    L = make(ctx)
+    try:
+        issue(ctx, L)
+    except G.GdagError as e:
+        assert e.remaining[0] == e.issued
+        if e.issued > 0:  # the first unit ran, with the second square and the sum
+            assert not {0, 3, 5} & set(e.remaining)
+        issue(ctx, [L[j] for j in e.remaining])
+        # no unit is missing and none ran twice, but for the one that failed, if it
+        # came as far as its launch
+        assert ctx.stats()["launches"] - launches in (0, 1)
+    ctx.sync()
+    assert ctx.stats()["active"] == 0
+    ctx.close()
