@@ -199,9 +199,9 @@ typedef struct {
     int32_t type;    /* GDAG_OP_*                                            */
     int32_t stream;  /* pool index, -1 for host ops                          */
     int32_t event;   /* event slot for RECORD/WAIT/HOST_WAIT, else -1        */
-    int32_t beside;  /* COPY_*: 1 if kernels on other streams of the context
-                        may run at the same time (the copy is then left to a
-                        copy engine), else 0                                 */
+    int32_t beside;  /* COPY_*: 1 if kernels, or more than one copy, on other
+                        streams of the context may run at the same time (the
+                        copy is then left to a copy engine), else 0          */
     int64_t node;    /* node the op belongs to, -1 if none                   */
 } gdag_op;
 

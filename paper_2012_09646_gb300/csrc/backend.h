@@ -39,7 +39,7 @@ class Backend {
     virtual int launch(const KernelEntry &k, const LaunchArgs &a, void *s) = 0;
     virtual int launch_fused(const KernelEntry &k, const LaunchArgs *a, int count, void *s) = 0;
     virtual int launch_merged(const Merge &m, const LaunchArgs *const *a, const char *name, void *s) = 0;
-    // beside: kernels on other streams may run at the same time
+    // beside: kernels, or more than one copy, on other streams may run at the same time
     virtual int copy_h2d(void *dst, const void *src, size_t bytes, bool beside, void *s) = 0;
     virtual int copy_d2h(void *dst, const void *src, size_t bytes, bool beside, void *s) = 0;
     virtual int external(void (*fn)(void *, void *), void *user, void *s) = 0;

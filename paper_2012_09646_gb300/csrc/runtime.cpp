@@ -250,9 +250,13 @@ struct Ctx {
     {
         return n.kind == GDAG_NODE_HOST_WRITE || n.kind == GDAG_NODE_HOST_READ || n.kind == GDAG_NODE_HOST_PREFETCH;
     }
-    // Kernels that a copy on stream s does not follow may be running (they are
-    // not known to be complete).
-    bool kernels_beside(int32_t s) const { return active_kernels > streams[(size_t)s].kernels; }
+    // Work that a copy on stream s does not follow may be running (it is not known
+    // to be complete): a kernel, or more than one copy.
+    bool work_beside(int32_t s) const
+    {
+        const StreamState &ss = streams[(size_t)s];
+        return active_kernels > ss.kernels || (active_count - active_kernels) - (ss.active - ss.kernels) > 1;
+    }
 
     // Mark one active node inactive: its event slot and its stream's share
     // are released.  Returns false if it was not active.
@@ -1279,7 +1283,7 @@ int gdag_array_write(gdag_ctx *c, gdag_array a, const void *src, size_t off, siz
     int32_t st;
     r = c->place(id, &st);
     if (r) return c->drop_failed(id, r);
-    const bool beside = c->kernels_beside(st);
+    const bool beside = c->work_beside(st);
     c->log_op(GDAG_OP_COPY_H2D, st, -1, id, beside);
     ++c->st.copies;
     r = c->be->copy_h2d(static_cast<char *>(s->dev) + off, view, bytes, beside, c->streams[(size_t)st].handle);
@@ -1323,7 +1327,7 @@ int gdag_array_read(gdag_ctx *c, gdag_array a, void *dst, size_t off, size_t byt
         int32_t st;
         r = c->place(id, &st);
         if (r) return c->drop_failed(id, r);
-        const bool beside = c->kernels_beside(st);
+        const bool beside = c->work_beside(st);
         c->log_op(GDAG_OP_COPY_D2H, st, -1, id, beside);
         ++c->st.copies;
         r = c->be->copy_d2h(view, static_cast<char *>(s->dev) + off, bytes, beside, c->streams[(size_t)st].handle);
@@ -1373,7 +1377,7 @@ int gdag_array_prefetch_host(gdag_ctx *c, gdag_array a, size_t off, size_t bytes
     int32_t st;
     r = c->place(id, &st);
     if (r) return c->drop_failed(id, r);
-    const bool beside = c->kernels_beside(st);
+    const bool beside = c->work_beside(st);
     c->log_op(GDAG_OP_COPY_D2H, st, -1, id, beside);
     ++c->st.copies;
     r = c->be->copy_d2h(static_cast<char *>(s->host) + off, static_cast<char *>(s->dev) + off, bytes, beside,

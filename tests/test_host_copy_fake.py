@@ -69,3 +69,17 @@ def test_serial_policies_have_one_stream():
     ctx.write(y)
     assert copies(ctx) == [(1, 0)]
     ctx.close()
+
+
+def test_copies_beside_several_copies():
+    """Copies by kernels share the link; those by an engine come one after another, so
+    that what follows the first overlaps the others: from the third on, by an engine."""
+    ctx, a = make()
+    a += [ctx.array(dev=(i + 9) << 24, nbytes=400) for i in range(4)]
+    for x in a:
+        ctx.write(x)
+    assert [b for _, b in copies(ctx)] == [0, 0] + [1] * 6
+    ctx.sync()
+    ctx.write(a[0])
+    assert copies(ctx)[-1][1] == 0
+    ctx.close()
