@@ -482,7 +482,10 @@ int gdag_launch_external(gdag_ctx *ctx, void (*fn)(void *stream, void *user),
  * and completes as a whole, so the streams and waits, and the numbering of
  * the nodes inside the call, may differ from the single calls'.  A launch
  * joins a unit only if every launch it would overtake touches nothing that it
- * writes and writes nothing that it touches.  If a unit fails, all its
+ * writes and writes nothing that it touches.  Launches that are merely
+ * independent join only if none is held back by it: their unfinished parents
+ * must be on the same streams (host writes of up to 1 MB do not count for the
+ * kernels of HITS).  If a unit fails, all its
  * members fail: *issued counts the elements before its first one.  After a
  * failure at element f = *issued, an element j > f was issued (by an earlier
  * unit) if and only if nodes_out[j] >= 0 and nodes_out[f] is -1 or greater than

@@ -71,13 +71,18 @@ struct RunLaunch {
 class Run {
   public:
     // The kernel of the run's launch j; null past the run's end.
-    virtual const KernelEntry *kernel(int j) = 0;
+    const KernelEntry *kernel(int j) { return j < known_ ? kernel_[j] : look(j); }
     // Launch j, resolved and validated with those before it; null if the run ends
     // before.  Valid for this asking of the rule.
-    virtual const RunLaunch *at(int j) = 0;
+    const RunLaunch *at(int j) { return j < ready_ ? launch_[j] : resolve_to(j); }
 
   protected:
     ~Run() = default;
+    virtual const KernelEntry *look(int j) = 0;
+    virtual const RunLaunch *resolve_to(int j) = 0;
+    int known_ = 0, ready_ = 0;
+    const KernelEntry *kernel_[kMaxRun];
+    const RunLaunch *launch_[kMaxRun];
 };
 
 // As LauncherFn, over the members' arguments.
@@ -85,6 +90,11 @@ typedef int (*MergeLaunchFn)(const LaunchArgs *const *m, int count, void *stream
 struct Merge {
     int count = 0;
     int member[kMaxRun];  // indices into the run, in the order the launcher wants them
+    // The first `apart` members need nothing from one another: on streams of their
+    // own each would start as soon as its own inputs are there, and the runtime parts
+    // them where that differs.  Host writes of up to waits_for bytes do not count.
+    int apart = 0;
+    size_t waits_for = 0;
     MergeLaunchFn launch = nullptr;
 };
 typedef bool (*MergeFn)(Run &run, Merge &out);

@@ -31,6 +31,7 @@
 // Conditioning: C is a difference of two terms of size ~S, so for
 // sigma sqrt(T) well below 1e-2 an fp32 price near the strike carries an
 // error of a few ulp of S, whatever the evaluation.
+#include <algorithm>
 #include <cmath>
 #include <vector>
 
@@ -265,18 +266,21 @@ int launch_bs(const LaunchArgs &a, void *s)
     return cudaGetLastError();
 }
 
-template <int CAP> int fused_bs_cap(const LaunchArgs *a, int count, void *s)
+// member(i): the arguments of member i.
+template <int CAP, class Member> int fused_bs_cap(const Member &member, int count, void *s)
 {
     for (int off = 0; off < count; off += CAP) {
         BsFused<CAP> t;
         t.count = count - off < CAP ? count - off : CAP;
         t.start[0] = 0;
         for (int m = 0; m < t.count; ++m) {
-            const LaunchArgs &la = a[off + m];
+            const LaunchArgs &la = member(off + m);
             t.S[m] = la.p<float>(0);
             t.C[m] = la.p<float>(1);
             t.n[m] = la.i64(2);
-            t.c[m] = bs_const(la);
+            // books of one program mostly share K, r, sigma and T
+            const bool same = m > 0 && std::equal(la.val + 3, la.val + 7, member(off + m - 1).val + 3);
+            t.c[m] = same ? t.c[m - 1] : bs_const(la);
             t.start[m + 1] = t.start[m] + ceil_div(t.n[m], kBsChunk);
         }
         const int64_t total = t.start[t.count];
@@ -290,16 +294,19 @@ template <int CAP> int fused_bs_cap(const LaunchArgs *a, int count, void *s)
     return cudaSuccess;
 }
 
+template <class Member> int fused_bs_any(const Member &member, int count, void *s)
+{
+    return count <= kFuseSmall ? fused_bs_cap<kFuseSmall>(member, count, s) : fused_bs_cap<kFuseTable>(member, count, s);
+}
+
 int fused_bs(const LaunchArgs *a, int count, void *s)
 {
-    return count <= kFuseSmall ? fused_bs_cap<kFuseSmall>(a, count, s) : fused_bs_cap<kFuseTable>(a, count, s);
+    return fused_bs_any([=](int i) -> const LaunchArgs & { return a[i]; }, count, s);
 }
 
 int launch_bs_run(const LaunchArgs *const *m, int count, void *s)
 {
-    LaunchArgs a[kMaxRun];
-    for (int i = 0; i < count; ++i) a[i] = *m[i];
-    return fused_bs(a, count, s);
+    return fused_bs_any([=](int i) -> const LaunchArgs & { return *m[i]; }, count, s);
 }
 
 // Independent consecutive bs_call launches of up to kBsMergeMax options each
@@ -326,6 +333,7 @@ bool merge_bs(Run &run, Merge &out)
         if (!apart) break;
         out.member[out.count++] = i;
     }
+    out.apart = out.count;
     out.launch = launch_bs_run;
     return out.count > 1;
 }

@@ -832,7 +832,7 @@ template <MergeLaunchFn LAUNCH> bool merge_branches(Run &run, Merge &out)
         if (!run.at(j)) return false;
         const RunLaunch &g = *run.at(j);
         if (items(f.a) + items(g.a) > INT32_MAX / 2 || !apart(f, g)) return false;
-        out.count = 2;
+        out.count = out.apart = 2;
         out.member[0] = 0;
         out.member[1] = j;
         out.launch = LAUNCH;

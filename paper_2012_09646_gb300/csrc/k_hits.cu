@@ -716,6 +716,11 @@ int launch_seg_scale(const LaunchArgs &a, void *s)
 // graphs the two branches on two streams are the quicker form where one program
 // has the device (1e6 rows 287 us against 314, 1e7 2160 against 2234): a branch's
 // norm and scaling run beside the other's product.
+// A pair waits for short host writes of either: the first products of a program
+// whose vectors the host writes would otherwise part its branches to the end (five
+// iterations with the writes and the reads, parted and merged: 20000 vertices 180
+// and 163 us, 156250 248 and 238; 300000, 1.2 MB each, 285 and 281).
+constexpr size_t kWaitsFor = (size_t)1 << 20;
 template <MergeLaunchFn LAUNCH> bool merge_two(Run &run, Merge &out)
 {
     const RunLaunch &f = *run.at(0);
@@ -738,7 +743,8 @@ template <MergeLaunchFn LAUNCH> bool merge_two(Run &run, Merge &out)
                 if (f.array[p] >= 0 && f.array[p] == g.array[q])
                     apart = apart && f.k->spec[p].mode == GDAG_MODE_IN && g.k->spec[q].mode == GDAG_MODE_IN;
         if (!apart) return false;
-        out.count = 2;
+        out.count = out.apart = 2;
+        out.waits_for = kWaitsFor;
         out.member[0] = 0;
         out.member[1] = j;
         out.launch = LAUNCH;

@@ -639,7 +639,7 @@ bool merge_scores(Run &run, Merge &out)
         for (int i = 0; i < 3; ++i)
             apart = apart && f.array[i] != s0 && f.array[i] != s1 && g.array[i] != s0 && g.array[i] != s1;
         if (!apart) continue;
-        out.count = 2;
+        out.count = out.apart = 2;
         out.member[0] = 0;
         out.member[1] = j;
         out.launch = launch;

@@ -62,6 +62,7 @@ struct Node {
     bool active = false;
     bool first_child_taken = false;
     uint32_t parent_off = 0, parent_cnt = 0;
+    uint32_t bytes = 0;       // of a host write (the largest value for any above)
     int64_t parent_of = -1;   // last element that took this node as a parent
 };
 
@@ -97,13 +98,34 @@ struct Access {
 
 // A launch element of a gdag_issue call as the merge rules see it.
 struct Resolved {
-    int32_t elem = -1;
     bool ok;
     gdag::RunLaunch l;
     Access acc[gdag::kMaxArgs];
     int nacc;
 };
+// Those of one call, element i in place i mod kResolvedRing.
 constexpr int kResolvedRing = 64;
+struct ResolvedRing {
+    uint64_t call = 0;  // gdag_issue calls so far
+    struct {
+        uint64_t call = 0;
+        int32_t elem = -1;
+    } tag[kResolvedRing];
+    std::unique_ptr<Resolved[]> place;  // made at the first use
+    Resolved *find(int32_t i)
+    {
+        const size_t k = (size_t)i % kResolvedRing;
+        return tag[k].call == call && tag[k].elem == i ? &place[k] : nullptr;
+    }
+    Resolved &make(int32_t i)
+    {
+        const size_t k = (size_t)i % kResolvedRing;
+        if (!place) place.reset(new Resolved[kResolvedRing]);
+        tag[k].call = call;
+        tag[k].elem = i;
+        return place[k];
+    }
+};
 
 }  // namespace
 
@@ -145,7 +167,7 @@ struct Ctx {
     // scratch for one element or one call
     std::vector<int64_t> par, retire_stack, ext;
     std::vector<uint8_t> issued_early;
-    std::vector<Resolved> resolved;  // kResolvedRing once used
+    ResolvedRing ring;
 
     // stream capture (CUDA graphs of a repeated DAG shape)
     bool capturing = false;
@@ -271,8 +293,9 @@ struct Ctx {
         }
         if (n->stream >= 0) {
             StreamState &s = streams[(size_t)n->stream];
-            s.kernels -= !is_copy(*n);
-            active_kernels -= !is_copy(*n);
+            const int kernel = !is_copy(*n);
+            s.kernels -= kernel;
+            active_kernels -= kernel;
             if (--s.active == 0 && !s.queued) {
                 s.queued = true;
                 free_streams.push_back(n->stream);
@@ -458,6 +481,30 @@ struct Ctx {
         std::sort(par.begin(), par.end());
     }
 
+    // The streams (bit s mod 64) of the active parents that an element with accesses
+    // acc would have by infer's rule: *all of them, and those left when host writes
+    // of up to `waits_for` bytes do not count.
+    uint64_t parent_streams(const Access *acc, int n, size_t waits_for, uint64_t *all)
+    {
+        uint64_t counted = 0;
+        *all = 0;
+        auto take = [&](int64_t id) {
+            const Node *p = node(id);
+            if (!p || !p->active) return;
+            const uint64_t bit = (uint64_t)1 << (p->stream & 63);
+            *all |= bit;
+            if (p->kind != GDAG_NODE_HOST_WRITE || p->bytes > waits_for) counted |= bit;
+        };
+        for (int i = 0; i < n; ++i) {
+            const ArrayState &s = arrays[(size_t)acc[i].array];
+            if ((acc[i].bits & W_BIT) && !s.readers.empty())
+                for (int64_t r : s.readers) take(r);
+            else
+                take(s.writer);
+        }
+        return counted;
+    }
+
     // Append the node for element `id` (after infer()).
     void push_node(int32_t kind)
     {
@@ -610,15 +657,17 @@ struct Ctx {
     // Put the active node id on stream s as its last work.
     void attach(int64_t id, int32_t s)
     {
-        node(id)->stream = s;
+        Node *me = node(id);
+        me->stream = s;
         StreamState &ss = streams[(size_t)s];
         if (ss.queued) {  // taken from the FIFO by the LRU path: drop it
             ss.queued = false;
             free_streams.erase(std::find(free_streams.begin(), free_streams.end(), s));
         }
         ss.active++;
-        ss.kernels += !is_copy(*node(id));
-        active_kernels += !is_copy(*node(id));
+        const int kernel = !is_copy(*me);
+        ss.kernels += kernel;
+        active_kernels += kernel;
         ss.tail = id;
         ss.last_use = ++tick;
         if (opt.record_log == 1) node_log[node_log.size() - (size_t)(next_id() - id)].stream = s;
@@ -1280,6 +1329,7 @@ int gdag_array_write(gdag_ctx *c, gdag_array a, const void *src, size_t off, siz
     bool full = off == 0 && bytes == s->bytes;
     s->host_valid = s->host_valid || full;
     c->push_node(GDAG_NODE_HOST_WRITE);
+    c->node(id)->bytes = (uint32_t)std::min<size_t>(bytes, UINT32_MAX);
     int32_t st;
     r = c->place(id, &st);
     if (r) return c->drop_failed(id, r);
@@ -1401,14 +1451,12 @@ static bool elem_args_ok(const gdag_elem &e, int64_t nargs_total)
 
 // Launch element i for a merge rule: a built-in kernel with the automatic shape
 // and its signature's access modes, valid as it stands (with the context's last
-// error restored).  Resolved once a call: the ring holds the elements that the
-// runs since then looked at.
+// error restored).  Resolved once a call.
 static const Resolved &resolved(gdag_ctx *c, const gdag_elem *elems, int32_t i, const gdag_arg *args,
                                 int64_t nargs_total)
 {
-    Resolved &out = c->resolved[(size_t)i % kResolvedRing];
-    if (out.elem == i) return out;
-    out.elem = i;
+    if (const Resolved *x = c->ring.find(i)) return *x;
+    Resolved &out = c->ring.make(i);
     out.ok = false;
     const gdag_elem &e = elems[i];
     if (e.smem || e.grid.x || e.grid.y || e.grid.z || !elem_args_ok(e, nargs_total)) return out;
@@ -1446,45 +1494,52 @@ struct MergeRun final : gdag::Run {
     const gdag_arg *args;
     int64_t nargs_total;
     int32_t end;
-    int32_t elem[gdag::kMaxRun];              // the run's launches so far
-    int known = 1;
+    int32_t elem[gdag::kMaxRun];  // the run's launches so far
     bool ended = false;
-    const Resolved *r[gdag::kMaxRun];         // those resolved so far
-    int n = 0;
+    const Resolved *r[gdag::kMaxRun];  // those resolved so far
     gdag::Merge m;
     int order[gdag::kMaxRun];  // the members in the run's order
 
     MergeRun(gdag_ctx *ctx, const gdag_elem *e, int32_t ne, const gdag_arg *a, int64_t na, int32_t first)
-        : c(ctx), elems(e), args(a), nargs_total(na), end(std::min<int64_t>(ne, (int64_t)first + kResolvedRing))
+        : c(ctx), elems(e), args(a), nargs_total(na), end((int32_t)std::min<int64_t>(ne, (int64_t)first + kResolvedRing))
     {
         elem[0] = first;
+        kernel_[0] = &c->kernels[(size_t)e[first].kernel];
+        known_ = 1;
     }
-    const KernelEntry *kernel(int j) override
+    int n() const { return ready_; }
+    const KernelEntry *look(int j) override
     {
-        while (known <= j && !ended) {
-            int32_t i = elem[known - 1] + 1;
+        while (known_ <= j && !ended) {
+            int32_t i = elem[known_ - 1] + 1;
             while (i < end && !c->issued_early.empty() && c->issued_early[(size_t)i]) ++i;
-            if (known == gdag::kMaxRun || i >= end || elems[i].type != GDAG_ELEM_LAUNCH || elems[i].kernel < 0 ||
-                (size_t)elems[i].kernel >= c->kernels.size() || !c->kernels[(size_t)elems[i].kernel].launcher)
+            const KernelEntry *k = nullptr;
+            if (known_ < gdag::kMaxRun && i < end && elems[i].type == GDAG_ELEM_LAUNCH && elems[i].kernel >= 0 &&
+                (size_t)elems[i].kernel < c->kernels.size())
+                k = &c->kernels[(size_t)elems[i].kernel];
+            if (k && k->launcher) {
+                elem[known_] = i;
+                kernel_[known_++] = k;
+            } else {
                 ended = true;
-            else
-                elem[known++] = i;
+            }
         }
-        return j < known ? &c->kernels[(size_t)elems[elem[j]].kernel] : nullptr;
+        return j < known_ ? kernel_[j] : nullptr;
     }
-    const gdag::RunLaunch *at(int j) override
+    const gdag::RunLaunch *resolve_to(int j) override
     {
-        while (n <= j) {
-            if (!kernel(n)) return nullptr;
-            const Resolved &x = resolved(c, elems, elem[n], args, nargs_total);
+        while (ready_ <= j) {
+            if (!kernel(ready_)) return nullptr;
+            const Resolved &x = resolved(c, elems, elem[ready_], args, nargs_total);
             if (!x.ok) {
-                known = n;
+                known_ = ready_;
                 ended = true;
                 return nullptr;
             }
-            r[n++] = &x;
+            r[ready_] = &x;
+            launch_[ready_++] = &x.l;
         }
-        return &r[j]->l;
+        return launch_[j];
     }
     const Access *acc(int j) const { return r[j]->acc; }
     int nacc(int j) const { return r[j]->nacc; }
@@ -1494,14 +1549,14 @@ struct MergeRun final : gdag::Run {
 static bool merge_legal(gdag_ctx *c, MergeRun &q)
 {
     const gdag::Merge &m = q.m;
-    if (m.count < 2 || m.count > q.n || !m.launch) return false;
+    if (m.count < 2 || m.count > q.n() || !m.launch) return false;
     bool in[gdag::kMaxRun] = {};
     for (int k = 0; k < m.count; ++k) {
-        if (m.member[k] < 0 || m.member[k] >= q.n || in[m.member[k]]) return false;
+        if (m.member[k] < 0 || m.member[k] >= q.n() || in[m.member[k]]) return false;
         in[m.member[k]] = true;
     }
     if (!in[0]) return false;
-    for (int j = 0, k = 0; j < q.n; ++j)
+    for (int j = 0, k = 0; j < q.n(); ++j)
         if (in[j]) q.order[k++] = j;
     // a member moves up past every launch between it and the first one
     for (int k = 1; k < m.count; ++k)
@@ -1531,6 +1586,28 @@ static bool merge_legal(gdag_ctx *c, MergeRun &q)
         for (int j = i + 1; j < ns; ++j)
             if ((span[i].written || span[j].written) && span[i].lo < span[j].hi && span[j].lo < span[i].hi) return false;
     return true;
+}
+
+// Whether the unit would hold members back, having left out those that it may.
+// Members that need nothing from one another would each start when its own parents
+// are done; as a unit they start together.  So each must have its active parents on
+// the streams that the first one's are on, and the first one no others.  Ten books
+// of 2e6 options written, priced and read, one a launch: 660 us; as one unit, which
+// waits for the last write, 932 (5e5 options: 227 and 280, 1000: 94 and 103).
+static bool held_back(gdag_ctx *c, MergeRun &q)
+{
+    gdag::Merge &m = q.m;
+    if (m.apart < 2 || c->active_count == 0) return false;
+    uint64_t all0, all;
+    const uint64_t first = c->parent_streams(q.acc(m.member[0]), q.nacc(m.member[0]), m.waits_for, &all0);
+    for (int k = 1; k < m.apart; ++k) {
+        const uint64_t own = c->parent_streams(q.acc(m.member[k]), q.nacc(m.member[k]), m.waits_for, &all);
+        if (!(first & ~all) && !(own & ~all0)) continue;
+        if (k == 1 || m.apart < m.count) return true;
+        m.count = m.apart = k;  // the members before it make a unit
+        return !merge_legal(c, q);
+    }
+    return false;
 }
 
 // Issue the members of q.m as one unit: every member is an element of its own
@@ -1613,10 +1690,7 @@ static int issue_each(gdag_ctx *c, const gdag_elem *elems, int32_t n, const gdag
     const bool merging = c->opt.policy == GDAG_POLICY_PARALLEL && !c->opt.trace && !c->poisoned;
     std::vector<uint8_t> &done = c->issued_early;  // elements issued as members of an earlier unit
     done.clear();
-    if (merging) {
-        c->resolved.resize(kResolvedRing);
-        for (Resolved &x : c->resolved) x.elem = -1;
-    }
+    ++c->ring.call;
     for (int32_t i = 0; i < n; ++i) {
         const gdag_elem &e = elems[i];
         if (!done.empty() && done[(size_t)i]) {
@@ -1626,7 +1700,7 @@ static int issue_each(gdag_ctx *c, const gdag_elem *elems, int32_t n, const gdag
         if (merging && e.type == GDAG_ELEM_LAUNCH && i + 1 < n && e.kernel >= 0 &&
             (size_t)e.kernel < c->kernels.size() && c->kernels[(size_t)e.kernel].merge) {
             MergeRun q(c, elems, n, args, nargs_total, i);
-            if (q.at(0) && q.r[0]->l.k->merge(q, q.m) && merge_legal(c, q)) {
+            if (q.at(0) && q.r[0]->l.k->merge(q, q.m) && merge_legal(c, q) && !held_back(c, q)) {
                 int64_t ids[gdag::kMaxRun];
                 const int r = issue_merged(c, q, elems, ids);
                 if (done.empty()) done.resize((size_t)n, 0);
@@ -1652,8 +1726,8 @@ static int issue_each(gdag_ctx *c, const gdag_elem *elems, int32_t n, const gdag
                 break;
             }
             const gdag_arg *a = e.nargs ? args + e.arg0 : nullptr;
-            const Resolved *x = merging ? &c->resolved[(size_t)i % kResolvedRing] : nullptr;
-            if (x && x->elem == i && x->ok)  // a rule has looked at it
+            const Resolved *x = c->ring.find(i);
+            if (x && x->ok)  // a rule has looked at it
                 r = launch_resolved(c, e.kernel, x->l.a, x->acc, x->nacc, &node);
             else if (e.type == GDAG_ELEM_LAUNCH)
                 r = gdag_launch(c, e.kernel, e.grid, e.block, (size_t)e.smem, a, e.nargs, &node);

@@ -386,3 +386,43 @@ def test_dl_program_equals_its_launches(n, h, w, classes, swap):
             got.append(out)
     for a, b in zip(*got):
         assert torch.equal(a.view(torch.int16) if a.dtype == bf else a, b.view(torch.int16) if b.dtype == bf else b)
+
+
+@pytest.mark.parametrize("late", [0, 1])
+def test_a_unit_waits_for_parents_on_busy_streams(late):
+    """The unit's inputs are made by kernels on two streams, one of them long, and
+    its members' results are used on others at once."""
+    n, m = 200_000, 10_000_000
+    g = torch.Generator(device="cuda").manual_seed(3)
+    S = [torch.rand(k, generator=g, device="cuda") * 90 + 10 for k in ((m, n) if late == 0 else (n, m))]
+    got = []
+    for policy, want in ((G.GDAG_POLICY_PARALLEL, 1), (G.GDAG_POLICY_SERIAL_ASYNC, 3)):
+        with G.Context(policy=policy) as ctx:
+            v = VecDag(ctx, n)
+            SA = [ctx.array(s) for s in S]
+            C = [torch.zeros_like(s) for s in S]
+            CA = [ctx.array(c) for c in C]
+            use = [ctx.array(t) for t in (torch.zeros(n, device="cuda"), torch.zeros(n, device="cuda"))]
+            keep = []
+            torch.cuda.synchronize()
+            for step in range(4):
+                for k, dst in ((0, v.X), (1, v.Y)):
+                    for _ in range(6):
+                        ctx.launch("bs_call", SA[k], CA[k], S[k].numel(), 60.0 + step, 0.1, 0.2, 1.0)
+                    # the first n prices into the unit's array, after all of them
+                    ctx.launch("unsharp", ctx.array(C[k][:n]), CA[k], dst, 0.0, n)
+                p = ctx.program()
+                p.launch("vec_square", v.X, n)
+                p.launch("vec_square", v.Y, n)
+                p.launch("vec_reduce_diff", v.X, v.Y, v.Z, v.S, n)
+                before = ctx.stats()["launches"]
+                p.issue()
+                assert ctx.stats()["launches"] - before == want
+                for a, b in zip((v.X, v.Y), use):
+                    ctx.launch("unsharp", a, a, b, 0.0, n)
+                ctx.sync()
+                keep += [t.clone() for t in (v.x, v.y, v.z, use[0].tensor, use[1].tensor)]
+            got.append(keep)
+    for a, b in zip(*got):
+        assert same_bits(a, b)
+    assert not torch.equal(got[0][0], got[0][5])  # the steps differ

@@ -475,3 +475,106 @@ def test_what_remains_after_a_failure_can_be_issued(fail):
     ctx.sync()
     assert ctx.stats()["active"] == 0
     ctx.close()
+
+
+BIG = (1 << 20) + 4  # bytes of a write that a pair of HITS launches does not wait for
+
+
+def books(ctx, count, nbytes=BIG):
+    at = itertools.count(1)
+    arr = lambda: ctx.array(dev=next(at) << 24, nbytes=nbytes)  # noqa: E731
+    return [(arr(), arr()) for _ in range(count)]
+
+
+def price(p, book):
+    p.launch("bs_call", *book, book[0].nbytes // 4, 60.0, 0.1, 0.2, 1.0)
+
+
+@pytest.mark.parametrize("count,written,nbytes,want", [
+    (2, [], BIG, 1), (2, [0], BIG, 2), (2, [1], BIG, 2), (2, [0, 1], BIG, 2),  # ready; a long write for either, or both
+    (2, [1], 400, 2), (10, range(10), 400, 10),                                # however short
+    (3, [2], BIG, 2), (3, [0], BIG, 2), (5, [2], BIG, 3),                      # the ready ones still merge
+])
+def test_independent_launches_do_not_wait_for_one_anothers_inputs(count, written, nbytes, want):
+    ctx = G.Context(backend="fake", record_log=True)
+    B = books(ctx, count, nbytes)
+    p = ctx.program()
+    for k in written:
+        p.write(B[k][0])
+    for b in B:
+        price(p, b)
+    p.issue()
+    assert ctx.stats()["launches"] == want
+    # every launch follows its own writes on their stream: nothing waits
+    assert not [o for o in ctx.ops() if o[0] == G.GDAG_OP_WAIT]
+    ctx.sync()
+    p = ctx.program()      # all known to be complete: one launch
+    for b in B:
+        price(p, b)
+    before = ctx.stats()["launches"]
+    p.issue()
+    assert ctx.stats()["launches"] - before == 1
+    p.issue()              # the books' parents are all on the unit's stream
+    assert ctx.stats()["launches"] - before == 2
+    ctx.close()
+
+
+def test_independent_launches_do_not_wait_for_one_anothers_kernels():
+    """Two chains on two streams stay two chains; one that reads both joins them."""
+    ctx = G.Context(backend="fake", record_log=True)
+    x, y, u, w = (ctx.array(dev=(i + 1) << 24, nbytes=400) for i in range(4))
+    n, m = ctx.array(dev=8 << 24, nbytes=4), ctx.array(dev=9 << 24, nbytes=4)
+    ctx.launch("vec_square", x, 100)
+    ctx.launch("vec_square", y, 100)
+    chain = [("scale", x, n, 100), ("scale", y, m, 100)]
+    assert issue(ctx, chain)[1] == 2 and issue(ctx, chain)[1] == 2
+    assert not [o for o in ctx.ops() if o[0] == G.GDAG_OP_WAIT]
+    ctx.launch("unsharp", x, y, u, 0.5, 100)          # waits for one of them
+    assert issue(ctx, [("scale", u, n, 100), ("scale", w, m, 100)])[1] == 2   # w is ready
+    ctx.sync()
+    assert issue(ctx, chain)[1] == 1 and issue(ctx, chain)[1] == 1
+    ctx.close()
+
+
+@pytest.mark.parametrize("n,want", [(1000, 3), (BIG // 4 - 1, 3), (BIG // 4, 6)])
+def test_hits_iterations_after_host_writes(n, want):
+    """The branches' vectors written by the host: short writes do not part them."""
+    ctx = G.Context(backend="fake", record_log=True)
+    at = itertools.count(1)
+    arr = lambda nb: ctx.array(dev=next(at) << 28, nbytes=nb)  # noqa: E731
+    sb, nnz = G.gdag_scratch_bytes, 2 * n
+    mats = [(arr(4 * (n + 1)), arr(4 * nnz), arr(4 * nnz)) for _ in range(2)]
+    part, car = ([arr(sb(k, n + nnz)) for _ in range(2)] for k in ("spmv_partition", "spmv_csr"))
+    V, N, S = [arr(4 * n) for _ in range(4)], [arr(4) for _ in range(2)], [arr(sb("l2norm", n)) for _ in range(2)]
+    ctx.write(V[0])
+    ctx.write(V[1])
+    cur, nxt = (0, 1), (2, 3)
+    for it in range(3):
+        seq = [("spmv_csr", *mats[1], V[cur[1]], part[1], V[nxt[0]], car[1], n, nnz),
+               ("spmv_csr", *mats[0], V[cur[0]], part[0], V[nxt[1]], car[0], n, nnz)]
+        seq += [("l2norm", V[nxt[k]], N[k], S[k], n) for k in range(2)]
+        seq += [("scale", V[nxt[k]], N[k], n) for k in range(2)]
+        # (later iterations of the parted branches meet again at the norms' scalars)
+        assert issue(ctx, seq)[1] == want or (it > 0 and want > 3)
+        cur, nxt = nxt, cur
+    ctx.close()
+
+
+def test_convolutions_do_not_wait_for_one_anothers_images():
+    n, h, w = 8, 256, 256
+
+    def dl(ctx, write):
+        at = itertools.count(1)
+        a = lambda nb: ctx.array(dev=next(at) << 28, nbytes=nb)  # noqa: E731
+        X = [a(2 * 3 * n * h * w) for _ in range(2)]
+        P, E = [a(2 * 64 * n * h * w // 4) for _ in range(2)], [a(4 * 64 * n) for _ in range(2)]
+        seq = [("conv3x3_relu_pool", X[k], a(2 * 64 * 27), a(256), P[k], a(4), n, h, w) for k in range(2)]
+        seq += [("avgpool_global", P[k], E[k], 64 * n, h * w // 4) for k in range(2)]
+        seq.append(("concat_dense", *E, a(4 * 128 * 10), a(40), a(40 * n), n, 64, 10))
+        for k in write:
+            ctx.write(X[k])
+        return issue(ctx, seq)[1]
+    for write, want in (([], 1), ([0], 5), ([1], 5), ([0, 1], 5)):
+        ctx = G.Context(backend="fake")
+        assert dl(ctx, write) == want, write
+        ctx.close()
