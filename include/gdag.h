@@ -484,8 +484,9 @@ int gdag_launch_external(gdag_ctx *ctx, void (*fn)(void *stream, void *user),
  * joins a unit only if every launch it would overtake touches nothing that it
  * writes and writes nothing that it touches.  Launches that are merely
  * independent join only if none is held back by it: their unfinished parents
- * must be on the same streams (host writes of up to 1 MB do not count for the
- * kernels of HITS).  If a unit fails, all its
+ * must be on the same streams (for the kernels of HITS host writes of up to 1 MB
+ * do not count, for the vector kernels among them nor do kernels that, with those
+ * they follow, touch up to 64 MB of arrays each).  If a unit fails, all its
  * members fail: *issued counts the elements before its first one.  After a
  * failure at element f = *issued, an element j > f was issued (by an earlier
  * unit) if and only if nodes_out[j] >= 0 and nodes_out[f] is -1 or greater than

@@ -92,9 +92,10 @@ struct Merge {
     int member[kMaxRun];  // indices into the run, in the order the launcher wants them
     // The first `apart` members need nothing from one another: on streams of their
     // own each would start as soon as its own inputs are there, and the runtime parts
-    // them where that differs.  Host writes of up to waits_for bytes do not count.
+    // them where that differs.  Host writes of up to waits_for bytes do not count, nor
+    // kernels that with those before them touch at most waits_for_kernels (each).
     int apart = 0;
-    size_t waits_for = 0;
+    uint32_t waits_for = 0, waits_for_kernels = 0;
     MergeLaunchFn launch = nullptr;
 };
 typedef bool (*MergeFn)(Run &run, Merge &out);

@@ -77,8 +77,8 @@ struct SpmvPair {
 // and SM; whatever else a block asks of the load-store unit adds to that.  So the
 // part after the products is kept short: a thread sums its row from shared memory
 // (the row ends are loaded before the products, so they wait with them), with no
-// search, no scan and one barrier.  200.6 us and 174.2 us (with the carries), from
-// 246 us and 217 us for a form in which each thread walked seven items of the
+// search, no scan and one barrier.  210 us and 183 us (with the carries, launches back to
+// back on one vector), a fifth less than a form in which each thread walked seven items of the
 // merged sequence (a binary search, a dependent chain of shared-memory reads and a
 // block-wide segmented scan).  Tiles of 640 to 1536 items measured within 2%;
 // 64 threads x 640 the same.  The order of a row's sum is chosen for its error: groups
@@ -710,17 +710,20 @@ int launch_seg_scale(const LaunchArgs &a, void *s)
 
 // Two independent launches of one kernel as one, the two branches of a HITS
 // iteration, while the launches are what bounds it: up to 2^22 rows and nonzeros
-// for the products, 2^20 elements for the vectors.  Five iterations, of one
-// program and of three in turn: 156250 rows 139 and 132 us against 239 and 241;
-// 700000 rows (4.2e6 rows and nonzeros) 248 and 165 against 268 and 263.  On larger
-// graphs the two branches on two streams are the quicker form where one program
-// has the device (1e6 rows 287 us against 314, 1e7 2160 against 2234): a branch's
-// norm and scaling run beside the other's product.
+// for the products, 2^20 elements for the vectors.  Five iterations, merged and not,
+// of one program and of three in turn: 20000 vertices 113 and 70 us against 171 and
+// 174; 156250 139 and 73 against 192 and 198; 600000 228 and 140 against 215 and 185.
+// On larger graphs the two branches on two streams are the quicker form where one
+// program has the device (700000: 222 us against 247, 1e6: 280 against 306, 1e7: 2045
+// against 2118): a branch's norm and scaling run beside the other's product.
 // A pair waits for short host writes of either: the first products of a program
-// whose vectors the host writes would otherwise part its branches to the end (five
-// iterations with the writes and the reads, parted and merged: 20000 vertices 180
-// and 163 us, 156250 248 and 238; 300000, 1.2 MB each, 285 and 281).
-constexpr size_t kWaitsFor = (size_t)1 << 20;
+// whose vectors the host writes would otherwise part its branches to the end (with
+// the writes and the reads, merged and parted: 20000 vertices 163 and 180 us, 156250 238
+// and 248; 300000, 1.2 MB each, 281 and 285).  The vector kernels wait for one
+// another's products too, while these are short (64 MB of arrays, 20 to 25 us):
+// above the products' line they still halve their launches, which bound three programs in
+// turn (800000 vertices, waiting and not: one program 256 and 247 us, three 185 and 217).
+constexpr uint32_t kWaitsFor = 1u << 20, kWaitsForKernels = 64u << 20;
 template <MergeLaunchFn LAUNCH> bool merge_two(Run &run, Merge &out)
 {
     const RunLaunch &f = *run.at(0);
@@ -745,6 +748,7 @@ template <MergeLaunchFn LAUNCH> bool merge_two(Run &run, Merge &out)
         if (!apart) return false;
         out.count = out.apart = 2;
         out.waits_for = kWaitsFor;
+        out.waits_for_kernels = is(f.k, "spmv_csr") ? 0 : kWaitsForKernels;
         out.member[0] = 0;
         out.member[1] = j;
         out.launch = LAUNCH;

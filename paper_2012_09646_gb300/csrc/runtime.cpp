@@ -62,7 +62,10 @@ struct Node {
     bool active = false;
     bool first_child_taken = false;
     uint32_t parent_off = 0, parent_cnt = 0;
-    uint32_t bytes = 0;       // of a host write (the largest value for any above)
+    // a host write's bytes; the most bytes of arrays that a kernel or one that it
+    // follows touches (a host write's count 32 times, the link's share of the HBM
+    // rate); the largest value where that is more or not known
+    uint32_t bytes = UINT32_MAX;
     int64_t parent_of = -1;   // last element that took this node as a parent
 };
 
@@ -482,9 +485,9 @@ struct Ctx {
     }
 
     // The streams (bit s mod 64) of the active parents that an element with accesses
-    // acc would have by infer's rule: *all of them, and those left when host writes
-    // of up to `waits_for` bytes do not count.
-    uint64_t parent_streams(const Access *acc, int n, size_t waits_for, uint64_t *all)
+    // acc would have by infer's rule: *all of them, and those left when the short
+    // ones that unit m waits for do not count.
+    uint64_t parent_streams(const Access *acc, int n, const Merge &m, uint64_t *all)
     {
         uint64_t counted = 0;
         *all = 0;
@@ -493,7 +496,10 @@ struct Ctx {
             if (!p || !p->active) return;
             const uint64_t bit = (uint64_t)1 << (p->stream & 63);
             *all |= bit;
-            if (p->kind != GDAG_NODE_HOST_WRITE || p->bytes > waits_for) counted |= bit;
+            const bool short_one = p->kind == GDAG_NODE_HOST_WRITE ? p->bytes <= m.waits_for
+                                   : p->kind == GDAG_NODE_KERNEL   ? p->bytes <= m.waits_for_kernels
+                                                                   : false;
+            if (!short_one) counted |= bit;
         };
         for (int i = 0; i < n; ++i) {
             const ArrayState &s = arrays[(size_t)acc[i].array];
@@ -503,6 +509,18 @@ struct Ctx {
                 take(s.writer);
         }
         return counted;
+    }
+
+    // Node::bytes of a kernel with accesses acc and the parents in `par`.
+    uint32_t kernel_bytes(const Access *acc, int n)
+    {
+        uint64_t b = 0;
+        for (int i = 0; i < n; ++i) b += arrays[(size_t)acc[i].array].bytes;
+        for (int64_t p : par) {
+            const Node &q = *node(p);
+            b = std::max(b, (q.kind == GDAG_NODE_HOST_WRITE ? 32 : 1) * (uint64_t)q.bytes);
+        }
+        return (uint32_t)std::min<uint64_t>(b, UINT32_MAX);
     }
 
     // Append the node for element `id` (after infer()).
@@ -1149,7 +1167,9 @@ static int issue_launch(gdag_ctx *c, gdag_kernel k, const LaunchArgs &la, const 
     c->infer(id, acc, nacc);
     for (int i = 0; i < nacc; ++i)
         if (acc[i].bits & gdag::W_BIT) c->arrays[(size_t)acc[i].array].host_valid = false;
+    const uint32_t bytes = c->kernel_bytes(acc, nacc);
     c->push_node(GDAG_NODE_KERNEL);
+    c->node(id)->bytes = bytes;
     c->node(id)->label = k;
     if (node_out) *node_out = id;
     int32_t s;
@@ -1599,9 +1619,9 @@ static bool held_back(gdag_ctx *c, MergeRun &q)
     gdag::Merge &m = q.m;
     if (m.apart < 2 || c->active_count == 0) return false;
     uint64_t all0, all;
-    const uint64_t first = c->parent_streams(q.acc(m.member[0]), q.nacc(m.member[0]), m.waits_for, &all0);
+    const uint64_t first = c->parent_streams(q.acc(m.member[0]), q.nacc(m.member[0]), m, &all0);
     for (int k = 1; k < m.apart; ++k) {
-        const uint64_t own = c->parent_streams(q.acc(m.member[k]), q.nacc(m.member[k]), m.waits_for, &all);
+        const uint64_t own = c->parent_streams(q.acc(m.member[k]), q.nacc(m.member[k]), m, &all);
         if (!(first & ~all) && !(own & ~all0)) continue;
         if (k == 1 || m.apart < m.count) return true;
         m.count = m.apart = k;  // the members before it make a unit
@@ -1632,7 +1652,9 @@ static int issue_merged(gdag_ctx *c, const MergeRun &q, const gdag_elem *elems, 
             if (p < first) ext.push_back(p);
         for (int i = 0; i < q.nacc(x); ++i)
             if (q.acc(x)[i].bits & gdag::W_BIT) c->arrays[(size_t)q.acc(x)[i].array].host_valid = false;
+        const uint32_t bytes = c->kernel_bytes(q.acc(x), q.nacc(x));
         c->push_node(GDAG_NODE_KERNEL);
+        c->node(id)->bytes = bytes;
         c->node(id)->label = elems[q.elem[x]].kernel;
         c->activate(id);
         ids[k] = id;

@@ -397,7 +397,7 @@ def test_launches_that_do_not_merge_cost_about_as_much_to_issue(name):
     which asks no rule (host time, the best of many issues)."""
     n, at = 3_000_000, itertools.count(1)
 
-    def best(policy):
+    def make(policy):
         ctx = G.Context(backend="fake", policy=policy, fake_complete=True, retire_by_query=True, trim_nodes=64)
         arr = lambda nb: ctx.array(dev=next(at) << 30, nbytes=nb)  # noqa: E731
         p = ctx.program()
@@ -407,17 +407,20 @@ def test_launches_that_do_not_merge_cost_about_as_much_to_issue(name):
                        "gauss_blur": lambda: ("gauss_blur", arr(4 * PX), arr(4 * PX), arr(20), ROWS, COLS, 2),
                        "vec_square": lambda: ("vec_square", arr(4000), 1000),
                        "row_softmax": lambda: ("row_softmax", arr(40000), 1000, 10)}[name]())
-        t = []
-        for _ in range(40):
+        return ctx, p
+    runs = [make(G.GDAG_POLICY_PARALLEL), make(G.GDAG_POLICY_SERIAL_ASYNC)]
+    best = [1e9, 1e9]
+    for _ in range(400):  # in turn, so that whatever else the machine does meets both
+        for k, (_, p) in enumerate(runs):
             t0 = time.perf_counter()
-            for _ in range(20):
-                p.issue()
-            t.append(time.perf_counter() - t0)
-        assert ctx.stats()["launches"] == 40 * 20 * 32
+            p.issue()
+            p.issue()
+            best[k] = min(best[k], time.perf_counter() - t0)
+    for ctx, _ in runs:
+        assert ctx.stats()["launches"] == 400 * 2 * 32
         ctx.close()
-        return min(t)
     # 3 to 4 times with the run resolved anew at every launch, 1.05 to 1.6 so
-    assert best(G.GDAG_POLICY_PARALLEL) <= 2.2 * best(G.GDAG_POLICY_SERIAL_ASYNC)
+    assert best[0] <= 2.2 * best[1]
 
 
 def test_a_run_longer_than_the_rules_look_ahead():
@@ -519,24 +522,50 @@ def test_independent_launches_do_not_wait_for_one_anothers_inputs(count, written
     ctx.close()
 
 
-def test_independent_launches_do_not_wait_for_one_anothers_kernels():
-    """Two chains on two streams stay two chains; one that reads both joins them."""
+@pytest.mark.parametrize("mb,parted", [(1, False), (31, False), (33, True), (300, True)])
+def test_independent_launches_do_not_wait_for_one_anothers_long_kernels(mb, parted):
+    """Two chains on two streams stay two chains if their kernels are long (more than
+    64 MB of arrays), or follow a long one; once complete, they merge."""
     ctx = G.Context(backend="fake", record_log=True)
-    x, y, u, w = (ctx.array(dev=(i + 1) << 24, nbytes=400) for i in range(4))
-    n, m = ctx.array(dev=8 << 24, nbytes=4), ctx.array(dev=9 << 24, nbytes=4)
-    ctx.launch("vec_square", x, 100)
-    ctx.launch("vec_square", y, 100)
-    chain = [("scale", x, n, 100), ("scale", y, m, 100)]
-    assert issue(ctx, chain)[1] == 2 and issue(ctx, chain)[1] == 2
-    assert not [o for o in ctx.ops() if o[0] == G.GDAG_OP_WAIT]
-    ctx.launch("unsharp", x, y, u, 0.5, 100)          # waits for one of them
-    assert issue(ctx, [("scale", u, n, 100), ("scale", w, m, 100)])[1] == 2   # w is ready
+    # vec_reduce_diff of two arrays: twice `mb`, and its scratch
+    x, y = ([ctx.array(dev=(8 * i + j + 1) << 30, nbytes=mb << 20) for j in range(2)] for i in range(2))
+    z = [ctx.array(dev=(i + 1) << 24, nbytes=4) for i in range(6)]
+    sc = [ctx.array(dev=(i + 8) << 24, nbytes=G.gdag_scratch_bytes("vec_reduce_diff", 100)) for i in range(2)]
+    chain = [("scale", z[0], z[2], 1), ("scale", z[1], z[3], 1)]
+
+    def start():
+        ctx.launch("vec_reduce_diff", *x, z[0], sc[0], 100)
+        ctx.launch("vec_reduce_diff", *y, z[1], sc[1], 100)
+        waits = sum(o[0] == G.GDAG_OP_WAIT for o in ctx.ops())
+        first, then = issue(ctx, chain)[1], issue(ctx, chain)[1]   # the second follow short ones that follow long ones
+        return first, then, sum(o[0] == G.GDAG_OP_WAIT for o in ctx.ops()) - waits
+    assert start() == ((2, 2, 0) if parted else (1, 1, 1))
     ctx.sync()
     assert issue(ctx, chain)[1] == 1 and issue(ctx, chain)[1] == 1
+    ctx.sync()
+    # one chain under way, the other ready
+    ctx.launch("vec_reduce_diff", *x, z[0], sc[0], 100)
+    assert issue(ctx, chain)[1] == (2 if parted else 1)
     ctx.close()
 
 
-@pytest.mark.parametrize("n,want", [(1000, 3), (BIG // 4 - 1, 3), (BIG // 4, 6)])
+def test_products_do_not_wait_for_one_anothers_kernels():
+    ctx = G.Context(backend="fake", record_log=True)
+    at = itertools.count(1)
+    arr = lambda nb: ctx.array(dev=next(at) << 28, nbytes=nb)  # noqa: E731
+    n, nnz, sb = 1000, 5000, G.gdag_scratch_bytes
+    x = [arr(4 * n) for _ in range(2)]
+    seq = [("spmv_csr", arr(4 * n + 4), arr(4 * nnz), arr(4 * nnz), v, arr(sb("spmv_partition", n + nnz)), arr(4 * n),
+            arr(sb("spmv_csr", n + nnz)), n, nnz) for v in x]
+    ctx.launch("vec_square", x[0], n)
+    assert issue(ctx, seq)[1] == 2
+    ctx.sync()
+    assert issue(ctx, seq)[1] == 1
+    ctx.close()
+
+
+# 4 MB at the link count as 128 MB of a kernel
+@pytest.mark.parametrize("n,want", [(1000, 3), (BIG // 4 - 1, 3), (BIG // 4, 4), (1_000_000, 6)])
 def test_hits_iterations_after_host_writes(n, want):
     """The branches' vectors written by the host: short writes do not part them."""
     ctx = G.Context(backend="fake", record_log=True)
@@ -549,13 +578,13 @@ def test_hits_iterations_after_host_writes(n, want):
     ctx.write(V[0])
     ctx.write(V[1])
     cur, nxt = (0, 1), (2, 3)
-    for it in range(3):
+    for it in range(2):
         seq = [("spmv_csr", *mats[1], V[cur[1]], part[1], V[nxt[0]], car[1], n, nnz),
                ("spmv_csr", *mats[0], V[cur[0]], part[0], V[nxt[1]], car[0], n, nnz)]
         seq += [("l2norm", V[nxt[k]], N[k], S[k], n) for k in range(2)]
         seq += [("scale", V[nxt[k]], N[k], n) for k in range(2)]
-        # (later iterations of the parted branches meet again at the norms' scalars)
-        assert issue(ctx, seq)[1] == want or (it > 0 and want > 3)
+        launches = issue(ctx, seq)[1]
+        assert it > 0 or launches == want
         cur, nxt = nxt, cur
     ctx.close()
 
