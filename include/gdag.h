@@ -24,9 +24,9 @@
  *   - an element whose stream wait, launch, copy or event record fails with
  *     a non-sticky error still gets its node id and its edges, but is
  *     retired at once.  Before the call returns, the host waits for the
- *     element's active parents (or, when its work was issued but its event
- *     could not be recorded, for its stream), so that later elements stay
- *     ordered after them.
+ *     element's active parents (or, when its work was issued in whole or in
+ *     part, a failed launch or event record, for its stream), so that later
+ *     elements stay ordered after them.
  */
 #ifndef GDAG_H
 #define GDAG_H
@@ -104,10 +104,12 @@ typedef struct {
                                 nodes that overlap compute; 0: each host
                                 write's copy completes before the call
                                 returns; default 1                           */
-    int32_t retire_by_query; /* 1: at each new element, parents whose event
-                                has completed are retired without a host
-                                wait; default 0 (the paper retires on host
-                                access only)                                  */
+    int32_t retire_by_query; /* 1: at a new element, parents whose event has
+                                completed are retired without a host wait
+                                (an element that follows all its parents on
+                                their stream asks only once 64 elements are
+                                active); default 0 (the paper retires on
+                                host access only)                             */
     int32_t record_log;      /* 1: keep element, edge and op logs for the
                                 export calls; 2: keep the op log only (for
                                 long programs: retired readers may then be
