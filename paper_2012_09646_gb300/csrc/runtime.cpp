@@ -511,16 +511,20 @@ struct Ctx {
         return counted;
     }
 
-    // Node::bytes of a kernel with accesses acc and the parents in `par`.
-    uint32_t kernel_bytes(const Access *acc, int n)
+    // Node::bytes of a kernel: of its accesses acc alone, and with the parents in `ps`.
+    uint64_t array_bytes(const Access *acc, int n) const
     {
         uint64_t b = 0;
         for (int i = 0; i < n; ++i) b += arrays[(size_t)acc[i].array].bytes;
-        for (int64_t p : par) {
+        return b;
+    }
+    uint32_t kernel_bytes(uint64_t own, const std::vector<int64_t> &ps)
+    {
+        for (int64_t p : ps) {
             const Node &q = *node(p);
-            b = std::max(b, (q.kind == GDAG_NODE_HOST_WRITE ? 32 : 1) * (uint64_t)q.bytes);
+            own = std::max(own, (q.kind == GDAG_NODE_HOST_WRITE ? 32 : 1) * (uint64_t)q.bytes);
         }
-        return (uint32_t)std::min<uint64_t>(b, UINT32_MAX);
+        return (uint32_t)std::min<uint64_t>(own, UINT32_MAX);
     }
 
     // Append the node for element `id` (after infer()).
@@ -1167,7 +1171,7 @@ static int issue_launch(gdag_ctx *c, gdag_kernel k, const LaunchArgs &la, const 
     c->infer(id, acc, nacc);
     for (int i = 0; i < nacc; ++i)
         if (acc[i].bits & gdag::W_BIT) c->arrays[(size_t)acc[i].array].host_valid = false;
-    const uint32_t bytes = c->kernel_bytes(acc, nacc);
+    const uint32_t bytes = c->kernel_bytes(c->array_bytes(acc, nacc), c->par);
     c->push_node(GDAG_NODE_KERNEL);
     c->node(id)->bytes = bytes;
     c->node(id)->label = k;
@@ -1584,27 +1588,35 @@ static bool merge_legal(gdag_ctx *c, MergeRun &q)
             if (!in[j] && conflicting(q.acc(j), q.nacc(j), q.acc(x), q.nacc(x))) return false;
     // what a member writes shares no memory with any other array of the unit
     // (other handles may name the same memory: the members would no longer
-    // run one after another on it)
+    // run one after another on it): the arrays in the order of their addresses
     struct Span {
+        uintptr_t lo, hi;
         int32_t array;
         bool written;
-        uintptr_t lo, hi;
     } span[gdag::kMaxRun * gdag::kMaxArgs];
     int ns = 0;
     for (int k = 0; k < m.count; ++k)
         for (int x = 0, mem = q.order[k]; x < q.nacc(mem); ++x) {
             const Access &w = q.acc(mem)[x];
-            int i = 0;
-            while (i < ns && span[i].array != w.array) ++i;
-            if (i == ns) {
-                const ArrayState &st = c->arrays[(size_t)w.array];
-                span[ns++] = Span{w.array, false, (uintptr_t)st.dev, (uintptr_t)st.dev + st.bytes};
+            const ArrayState &st = c->arrays[(size_t)w.array];
+            const uintptr_t lo = (uintptr_t)st.dev;
+            const bool written = (w.bits & gdag::W_BIT) != 0;
+            int i = ns;
+            while (i > 0 && (span[i - 1].lo > lo || (span[i - 1].lo == lo && span[i - 1].array > w.array))) --i;
+            if (i > 0 && span[i - 1].array == w.array) {
+                span[i - 1].written = span[i - 1].written || written;
+                continue;
             }
-            span[i].written = span[i].written || (w.bits & gdag::W_BIT);
+            std::copy_backward(span + i, span + ns, span + ns + 1);
+            span[i] = Span{lo, lo + st.bytes, w.array, written};
+            ++ns;
         }
-    for (int i = 0; i < ns; ++i)
-        for (int j = i + 1; j < ns; ++j)
-            if ((span[i].written || span[j].written) && span[i].lo < span[j].hi && span[j].lo < span[i].hi) return false;
+    uintptr_t end = 0, end_written = 0;  // of the arrays so far, of the written ones among them
+    for (int i = 0; i < ns; ++i) {
+        if (span[i].lo < (span[i].written ? end : end_written)) return false;
+        end = std::max(end, span[i].hi);
+        if (span[i].written) end_written = std::max(end_written, span[i].hi);
+    }
     return true;
 }
 
@@ -1642,6 +1654,7 @@ static int issue_merged(gdag_ctx *c, const MergeRun &q, const gdag_elem *elems, 
     const LaunchArgs *la[gdag::kMaxRun];
     std::vector<int64_t> &ext = c->ext;  // active parents outside the unit
     ext.clear();
+    uint64_t bytes = 0;
     for (int k = 0; k < m.count; ++k) {
         const int x = q.order[k];
         la[k] = &q.r[m.member[k]]->l.a;
@@ -1652,9 +1665,8 @@ static int issue_merged(gdag_ctx *c, const MergeRun &q, const gdag_elem *elems, 
             if (p < first) ext.push_back(p);
         for (int i = 0; i < q.nacc(x); ++i)
             if (q.acc(x)[i].bits & gdag::W_BIT) c->arrays[(size_t)q.acc(x)[i].array].host_valid = false;
-        const uint32_t bytes = c->kernel_bytes(q.acc(x), q.nacc(x));
+        if (m.count == 2) bytes = std::max(bytes, c->array_bytes(q.acc(x), q.nacc(x)));
         c->push_node(GDAG_NODE_KERNEL);
-        c->node(id)->bytes = bytes;
         c->node(id)->label = elems[q.elem[x]].kernel;
         c->activate(id);
         ids[k] = id;
@@ -1662,6 +1674,10 @@ static int issue_merged(gdag_ctx *c, const MergeRun &q, const gdag_elem *elems, 
     std::sort(ext.begin(), ext.end());
     ext.erase(std::unique(ext.begin(), ext.end()), ext.end());
     c->par = ext;
+    if (m.count == 2) {  // longer units count as long (Node::bytes as it is made)
+        const uint32_t unit_bytes = c->kernel_bytes(bytes, ext);
+        for (int k = 0; k < m.count; ++k) c->node(ids[k])->bytes = unit_bytes;
+    }
     // a failure drops every member, as drop_failed drops one
     auto drop = [&](int rc, int32_t stream) {
         const std::string msg = c->last_error;
