@@ -1,19 +1,17 @@
-// Short copies between a pinned host view and device memory, by a kernel.
-// A copy engine moves the bytes as fast, but every hand-over between it and a
-// kernel costs microseconds (a semaphore between two engines), which a short DAG
-// that writes, computes and reads pays twice.  Two writes of B bytes on two
-// streams, a kernel, a read of 4 bytes and the host's wait, by the copy engines and
-// by kernels: 62.5 KB 25.0 and 19.3 us, 500 KB 30.5 and 22.4 us, 4 MB 66.9 and
-// 57.4 us (16-byte pieces).  Longer copies are bound by the host link either way and
-// stay with the copy engines.  So do copies beside kernels of the same context that
-// they do not follow: 4 MB by a kernel beside an iteration of HITS at 4e6 vertices
-// (166 us) add 16 us to it, by an engine nothing.  And copies beside more than one
-// other: kernels share the link, engines do one copy after another, so that what follows
-// the first overlaps the rest (ten writes, B&S launches and reads of 5e5 options
-// each: 225 us, 258 us with every write by a kernel).  The one-byte pieces of unaligned
-// copies end at 64 KB (write, kernel and 64-byte read of 1 MB 31.5 us, with the
-// write by an engine 24.3; of 4 MB 71.7 and 46; of 64 KB 19.6 either way);
-// four-byte ones take 24.4, 45.5 and 19.6 us.
+// Short copies between a pinned host view and device memory, by a kernel. A copy engine moves
+// the bytes as fast, but every hand-over between it and a kernel costs microseconds (a
+// semaphore between two engines), which a short DAG that writes, computes and reads pays
+// twice.  Two writes of B bytes on two streams, a kernel, a read of 4 bytes and the host's
+// wait, by the copy engines and by kernels: 62.5 KB 25.0 and 19.3 us, 500 KB 30.5 and 22.4 us,
+// 4 MB 66.9 and 57.4 us (16-byte pieces).  Longer copies are bound by the host link either way
+// and stay with the copy engines.  So do copies beside kernels of the same context that they
+// do not follow: 4 MB by a kernel beside an iteration of HITS at 4e6 vertices (166 us) add 16
+// us to it, by an engine nothing.  And copies beside more than one other: kernels share the
+// link, engines do one copy after another, so that what follows the first overlaps the rest
+// (ten writes, B&S launches and reads of 5e5 options each: 225 us, 258 us with every write by
+// a kernel).  The one-byte pieces of unaligned copies end at 64 KB (write, kernel and 64-byte
+// read of 1 MB 31.5 us, with the write by an engine 24.3; of 4 MB 71.7 and 46; of 64 KB 19.6
+// either way); four-byte ones take 24.4, 45.5 and 19.6 us.
 #include <cuda.h>  // pointer attributes (the query comes from the runtime's driver entry point)
 #include <cuda_runtime.h>
 

@@ -77,15 +77,18 @@ struct SpmvPair {
 // and SM; whatever else a block asks of the load-store unit adds to that.  So the
 // part after the products is kept short: a thread sums its row from shared memory
 // (the row ends are loaded before the products, so they wait with them), with no
-// search, no scan and one barrier.  210 us and 183 us (with the carries, launches back to
-// back on one vector), a fifth less than a form in which each thread walked seven items of the
-// merged sequence (a binary search, a dependent chain of shared-memory reads and a
-// block-wide segmented scan).  Tiles of 640 to 1536 items measured within 2%;
-// 64 threads x 640 the same.  The order of a row's sum is chosen for its error: groups
-// of four as a tree, four sums taking the groups in turn, the one to three
-// products left added to the smallest of these (Sums4).  Rows of k uniform products are then off
-// (root mean square, relative) by 0.89 to 1.01 times what chains of seven and a
-// tree give, for every k up to 64; groups added to one sum, by 1.3 to 1.7 times from 31.
+// search, no scan and one barrier.  210 us and 183 us (with the carries, launches
+// back to back on one vector), from 247 us and 227 us for a form in which each thread
+// walked seven items of the merged sequence (a binary search, a dependent chain of
+// shared-memory reads and a block-wide segmented scan).  Tiles of 640 to 1536 items
+// measured within 2%; 64 threads x 640 the same.  The order of a row's sum is chosen
+// for its error: groups of four as a tree, four sums taking the groups in turn, the
+// one to three products left added to the smallest of these (Sums4).  Rows of k
+// uniform products are then off (root mean square, relative) by 0.89 to 1.01 times
+// what chains of seven and a tree give, for every k up to 64; groups added to one sum,
+// by 1.3 to 1.7 times from 31, and 218 us and 201 us.  Five iterations of HITS at 1e7
+// vertices, mean of 60 graphs: a is off by 6.04e-8 (6.33e-8 in the seven-item form),
+// h by 4.54e-8 (4.90e-8).
 // col and val are streamed once (evict-first); x is gathered through L1 and L2: in
 // the transpose of a power-law graph the high-degree vertices recur (L2-only
 // gathers: 471 us).  More loads of a thread in flight before its products (two or
